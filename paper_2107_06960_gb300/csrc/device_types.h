@@ -81,7 +81,17 @@ struct MafatStageDev {
     int32_t n_pieces;     // pieces per channel block (1: the set stays resident across items)
     int32_t sb_off;       // offset into the scale / bias arrays
     int32_t lookahead;    // 1: a CTA takes its next item as soon as this stage's item is loaded
-    int64_t w32_off;      // element offset of the fp32 weights [cout][cin][k][k]
+    // fp32 plans (CUDA-core kernel).  A task's conv region is cut into groups of 8 neighbouring
+    // pixels of a row, nbx per row: row by row (row pair by row pair, the two rows of a pair
+    // alternating, where a pool follows), or in blocks of f32_groups rows x one group column
+    // (f32_rect).  An item is the groups (bx * 32768 + by) * f32_groups .. of that sequence x
+    // n_blk output channels.
+    int32_t f32_ct;       // output channels per thread (8, 4, 2 or 1)
+    int32_t f32_groups;   // groups per item (16; 8 with f32_ct = 1)
+    int32_t f32_rect;
+    int32_t f32_chunks;   // shared-memory chunks of the input channels (4 channels of a 3x3, 16 of a 1x1)
+    int64_t f32_w_off;    // element offset of the packed fp32 weights: [channel block][chunk][tap]
+                          // [channel of the chunk][n_blk], padding zero
     // How a task of this stage that reads the caller's input (NHWC [frames][H][W][cin]) gets its
     // A halo into shared memory (tensor-core kernel; other tasks read octet-planar buffers):
     //   MAFAT_IN_PLANAR: one 4-D box per chunk (cin == 8, whose NHWC is one octet plane, or a

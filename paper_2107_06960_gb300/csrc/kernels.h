@@ -42,8 +42,10 @@ struct MafatKParams {
 // instance with the on-chip 3x3 -> 1x1 chaining path (plans that have chain stages).
 cudaError_t mafat_launch_tc(const MafatKParams& p, const CUtensorMap& in_map, int grid, bool chain, cudaStream_t s);
 size_t mafat_tc_smem_bytes();
-// fp32 CUDA-core check kernel: same work list, same scheduler.
+// fp32 CUDA-core kernel: same task list, same scheduler.
 cudaError_t mafat_launch_fp32(const MafatKParams& p, int grid, cudaStream_t s);
+int mafat_fp32_ctas_per_sm();
+size_t mafat_fp32_smem_bytes();
 // NHWC [frames][h][w][c] -> octet-planar [frames][c8][h][w][8] (padded channels zero),
 // for element sizes of 2 (bf16) or 4 (fp32) bytes.
 cudaError_t mafat_launch_to_planar(const void* nhwc, void* planar, int frames, int h, int w, int c, int c8,

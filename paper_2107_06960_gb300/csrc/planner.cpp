@@ -252,6 +252,56 @@ int largest_nblk(int cout) {
 
 }  // namespace
 
+namespace {
+
+// Channels of one shared-memory chunk of the fp32 kernel.
+int f32_chunk_channels(int k) { return k == 3 ? 4 : 16; }
+
+// Items along a region of ch x cw conv pixels (one output-channel block).
+int f32_region_items(const MafatStageDev& s, int ch, int cw) {
+    const int gx = ceil_div(cw, 8), G = s.f32_groups;
+    return s.f32_rect ? ceil_div(ch, G) * gx : (int)(((int64_t)ch * gx + G - 1) / G);
+}
+
+// Shape of an fp32 stage's items.  A thread computes 8 pixels x f32_ct channels, the CTA's 128
+// threads f32_groups x 8 pixels x 8, 16, 32 or 64 channels.  A chunk of a 3x3 costs a warp about
+// 288 f32_ct FFMA issue slots and ~120 more of loads and bookkeeping, so wide items are the
+// efficient ones, but a stage runs in ceil(items / SMs) turns of an SM's four schedulers: the
+// shape of the least (turns x cost), wider ones first.
+void f32_shape(MafatStageDev& s, const Layer& L, const std::vector<TileInfo>& tiles, int l, const PlanConfig& cfg,
+               int n_ctas, PlanTables& t) {
+    s.f32_rect = cfg.rect_blocks ? 1 : 0;
+    double best = 0.0;
+    int best_ct = 0;
+    for (int ct : {8, 4, 2, 1}) {
+        MafatStageDev q = s;
+        q.f32_groups = ct == 1 ? 8 : 16;
+        const int nb = ct == 1 ? 16 : 8 * ct;
+        if (cfg.fixed_nblk > 0 && nb > std::max(16, cfg.fixed_nblk)) continue;
+        int64_t items = 0;
+        for (const TileInfo& ti : tiles) {
+            const Rect& r = ti.outs[l];
+            if (!r.empty()) items += f32_region_items(q, r.h(), r.w());
+        }
+        items *= ceil_div(L.c_out, nb);
+        const double cost = (double)((items + n_ctas - 1) / n_ctas) * (288.0 * ct + 120.0);
+        if (best_ct == 0 || cost < best) {
+            best = cost;
+            best_ct = ct;
+        }
+    }
+    s.f32_ct = best_ct;
+    s.f32_groups = best_ct == 1 ? 8 : 16;
+    s.n_blk = best_ct == 1 ? 16 : 8 * best_ct;
+    s.n_nblk = ceil_div(L.c_out, s.n_blk);
+    s.mb = 1;
+    s.f32_chunks = ceil_div(L.c_in, f32_chunk_channels(L.k));
+    s.f32_w_off = t.pack32_elems;
+    t.pack32_elems += (int64_t)s.n_nblk * s.f32_chunks * f32_chunk_channels(L.k) * L.k * L.k * s.n_blk;
+}
+
+}  // namespace
+
 std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, bool* unsupported) {
     *unsupported = false;
     const int n = (int)net.layers.size();
@@ -493,7 +543,6 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
             }
             s.w_off = t.weight_elems;
             t.weight_elems += (int64_t)s.n_nblk * s.n_chunks * s.n_bsteps * s.blob_elems;
-            s.w32_off = t.weight32_elems;
             t.weight32_elems += (int64_t)L.c_out * L.c_in * L.k * L.k;
             s.sb_off = (int)t.sb_elems;
             t.sb_elems += cout_pad;
@@ -503,6 +552,7 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                 s.chain_a_col = cout_pad;
                 s.chain_out_col = cout_pad + cout_pad / 2;
             }
+            if (cfg.dtype == 1) f32_shape(s, L, tiles[g], l, cfg, n_ctas, t);
             t.stages.push_back(s);
             stage_pool_layer.push_back(s.pool ? l + 1 : -1);
             if (s.pool) ++l;
@@ -690,8 +740,13 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                         tk.cx0 = cr.x0;
                         tk.ch = cr.h();
                         tk.cw = cr.w();
-                        tk.nby = st.flat ? ceil_div(tk.ch * st.cols_box, 128) : ceil_div(tk.ch, MAFAT_BLK_ROWS);
-                        tk.nbx = st.flat ? 1 : ceil_div(tk.cw, MAFAT_BLK_COLS);
+                        if (st.f32_ct > 0) {  // fp32: items of the region, group columns
+                            tk.nby = f32_region_items(st, tk.ch, tk.cw);
+                            tk.nbx = ceil_div(tk.cw, 8);
+                        } else {
+                            tk.nby = st.flat ? ceil_div(tk.ch * st.cols_box, 128) : ceil_div(tk.ch, MAFAT_BLK_ROWS);
+                            tk.nbx = st.flat ? 1 : ceil_div(tk.cw, MAFAT_BLK_COLS);
+                        }
                         if (s == t.stage_first[g]) {
                             tk.in_kind = g == 0 ? MAFAT_BUF_USER_IN : g == 1 ? MAFAT_BUF_CUT : MAFAT_BUF_MAP;
                             tk.in_tmap = g >= 2 ? stage_tmap[s] : -1;
@@ -769,7 +824,9 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                             tk.out_y0 = orr.y0;
                             tk.out_x0 = orr.x0;
                         }
-                        tk.n_items = (st.blk_halo ? ceil_div(tk.nby * tk.nbx, st.mb) : ceil_div(tk.nby, st.mb) * tk.nbx) *
+                        tk.n_items = (st.f32_ct > 0    ? tk.nby
+                                      : st.blk_halo ? ceil_div(tk.nby * tk.nbx, st.mb)
+                                                    : ceil_div(tk.nby, st.mb) * tk.nbx) *
                                      st.n_nblk;
                         TaskDep d;
                         int qi = (int)(q - w0);
@@ -804,8 +861,12 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                             const MafatStageDev& sw = t.stages[sx];
                             const double kk = (double)sw.k * sw.k;
                             t.executed_flops += 2.0 * cr.h() * cr.w() * (double)sw.cout * sw.cin * kk;
-                            t.issued_flops += 2.0 * tk.nby * tk.nbx * (double)(MAFAT_BLK_ROWS * MAFAT_BLK_COLS) *
-                                              (double)sw.n_nblk * sw.n_blk * sw.n_chunks * sw.n_bsteps * sw.kst * 16.0;
+                            if (st.f32_ct > 0)
+                                t.issued_flops += 2.0 * tk.nby * 8.0 * st.f32_groups * (double)sw.n_nblk * sw.n_blk *
+                                                  sw.f32_chunks * f32_chunk_channels(sw.k) * kk;
+                            else
+                                t.issued_flops += 2.0 * tk.nby * tk.nbx * (double)(MAFAT_BLK_ROWS * MAFAT_BLK_COLS) *
+                                                  (double)sw.n_nblk * sw.n_blk * sw.n_chunks * sw.n_bsteps * sw.kst * 16.0;
                         }
                     }
                 }
@@ -898,15 +959,43 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
         if (deps[ti].bump_ctr >= 0) group_items[deps[ti].bump_ctr] += t.tasks[ti].n_items;
     }
     // ---- items
+    auto make_item = [&](int ti, int nb, int by, int bx, int nbk) {
+        const TaskDep& d = deps[ti];
+        MafatItemDev it{};
+        it.task = ti;
+        it.stage = (int16_t)t.tasks[ti].stage;
+        it.by = (int16_t)by;
+        it.nbk = (int16_t)nbk;
+        it.bx = (int16_t)bx;
+        it.nb = (int16_t)nb;
+        it.flags = (ti == cfg.unpublished_task) ? 1 : 0;
+        it.dep0 = -1;
+        it.dep1 = -1;
+        it.extra_ctr = -1;
+        if (d.prev_task >= 0) {
+            it.dep0 = MAFAT_CTR_BASE + d.prev_task;
+            it.dep0_target = t.tasks[d.prev_task].n_items;
+        }
+        if (d.group_ctr >= 0) {
+            it.dep1 = t.frame_ctr_base + d.group_ctr;
+            it.dep1_target = group_items[d.group_ctr];
+        }
+        if (d.bump_ctr >= 0) it.extra_ctr = t.frame_ctr_base + d.bump_ctr;
+        return it;
+    };
     for (int ti = 0; ti < n_tasks; ++ti) {
         const MafatTaskDev& tk = t.tasks[ti];
         const MafatStageDev& st = t.stages[tk.stage];
-        const TaskDep& d = deps[ti];
         // channel-block major: consecutive items share a resident weight set; a task's block
         // rows are split evenly over ceil(nby / mb) items (9 rows at mb = 8 give 5 + 4, not
         // 8 + 1, whose 1-block item would pay a whole item's fixed cost for little work)
         // Per-block-halo stages pack the task's blocks, in column-major order, evenly into
         // ceil(blocks / mb) items whatever the block columns (`by` = first block, `bx` = 0).
+        if (st.f32_ct > 0) {
+            for (int nb = 0; nb < st.n_nblk; ++nb)
+                for (int b = 0; b < tk.nby; ++b) t.items.push_back(make_item(ti, nb, b & 32767, b >> 15, 1));
+            continue;
+        }
         const int n_blocks = tk.nby * tk.nbx;
         const int n_rows = st.blk_halo ? ceil_div(n_blocks, st.mb) : ceil_div(tk.nby, st.mb);
         const int n_cols = st.blk_halo ? 1 : tk.nbx;
@@ -915,27 +1004,7 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
             for (int ri = 0; ri < n_rows; ++ri)
                 for (int bx = 0; bx < n_cols; ++bx) {
                     const int by = ri * n_span / n_rows, by_end = (ri + 1) * n_span / n_rows;
-                    MafatItemDev it{};
-                    it.task = ti;
-                    it.stage = (int16_t)tk.stage;
-                    it.by = (int16_t)by;
-                    it.nbk = (int16_t)(by_end - by);
-                    it.bx = (int16_t)bx;
-                    it.nb = (int16_t)nb;
-                    it.flags = (ti == cfg.unpublished_task) ? 1 : 0;
-                    it.dep0 = -1;
-                    it.dep1 = -1;
-                    it.extra_ctr = -1;
-                    if (d.prev_task >= 0) {
-                        it.dep0 = MAFAT_CTR_BASE + d.prev_task;
-                        it.dep0_target = t.tasks[d.prev_task].n_items;
-                    }
-                    if (d.group_ctr >= 0) {
-                        it.dep1 = t.frame_ctr_base + d.group_ctr;
-                        it.dep1_target = group_items[d.group_ctr];
-                    }
-                    if (d.bump_ctr >= 0) it.extra_ctr = t.frame_ctr_base + d.bump_ctr;
-                    t.items.push_back(it);
+                    t.items.push_back(make_item(ti, nb, by, bx, by_end - by));
                 }
     }
     if (t.items.size() > (size_t)0x7fffffff) return "too many work items";
@@ -992,6 +1061,19 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
                                           : scratch_total;
     };
     for (const MafatStageDev& s : t.stages) {
+        if (t.cfg.dtype == 1) {
+            const Layer& L = net.layers[s.layer];
+            const bool shape = s.f32_ct == 1 ? s.n_blk == 16 && s.f32_groups == 8
+                                             : (s.f32_ct == 2 || s.f32_ct == 4 || s.f32_ct == 8) &&
+                                                   s.n_blk == 8 * s.f32_ct && s.f32_groups == 16;
+            if (!shape || s.n_nblk * s.n_blk < L.c_out || s.mb != 1) return "bad fp32 item shape";
+            if (s.f32_chunks * f32_chunk_channels(s.k) < L.c_in || s.f32_w_off % 4 != 0 || s.f32_w_off < 0 ||
+                s.f32_w_off + (int64_t)s.n_nblk * s.f32_chunks * f32_chunk_channels(s.k) * s.k * s.k * s.n_blk >
+                    t.pack32_elems)
+                return "fp32 weights outside the packed weights";
+            if (L.c_out % 8 != 0 || s.sb_off < 0 || s.sb_off + L.c_out > t.sb_elems) return "bad fp32 channels";
+            continue;
+        }
         if ((int64_t)s.chunk8 * s.rows_box * s.cols_box * 16 > MAFAT_A_STAGE_BYTES) return "A box exceeds its stage";
         if (s.set_bytes != s.n_chunks * s.n_bsteps * s.blob_elems * 2 || s.set_bytes % 16 != 0)
             return "bad weight set size";
@@ -1069,7 +1151,9 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
         const Layer& L = net.layers[s.layer];
         if (s.chained) return "a chained stage has a task";
         if (last_item[ti] - first_item[ti] + 1 != k.n_items) return "task items not contiguous";
-        if (s.flat ? (k.cw + s.k - 1 > s.cols_box || k.nbx != 1 || k.nby != ceil_div(k.ch * s.cols_box, 128))
+        if (t.cfg.dtype == 1) {
+            if (k.nbx != ceil_div(k.cw, 8) || k.nby != f32_region_items(s, k.ch, k.cw)) return "task items do not tile its conv rectangle";
+        } else if (s.flat ? (k.cw + s.k - 1 > s.cols_box || k.nbx != 1 || k.nby != ceil_div(k.ch * s.cols_box, 128))
                    : (k.nby != ceil_div(k.ch, MAFAT_BLK_ROWS) || k.nbx != ceil_div(k.cw, MAFAT_BLK_COLS)))
             return "task blocks do not tile its conv rectangle";
         // input buffer extent and coverage of every in-map tap of the conv rectangle
@@ -1111,7 +1195,10 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
         const MafatItemDev& it = t.items[i];
         const MafatTaskDev& k = t.tasks[it.task];
         const MafatStageDev& s = t.stages[k.stage];
-        if (s.blk_halo) {
+        if (t.cfg.dtype == 1) {
+            if (it.by < 0 || it.bx < 0 || it.bx * 32768 + it.by >= k.nby || it.nb < 0 || it.nb >= s.n_nblk)
+                return "fp32 item out of range";
+        } else if (s.blk_halo) {
             // a run of the task's blocks in column-major order
             if ((int64_t)k.nby * k.nbx > 32767 || it.bx != 0 || it.by < 0 || it.nb < 0 || it.nb >= s.n_nblk ||
                 it.nbk < 1 || it.nbk > s.mb || it.by + it.nbk > k.nby * k.nbx)
@@ -1121,7 +1208,7 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
                 return "item block out of range";
             if (it.nbk < 1 || it.nbk > s.mb || it.by + it.nbk > k.nby) return "item block count out of range";
         }
-        if (s.flat) {
+        if (s.flat && t.cfg.dtype == 0) {
             // every pixel the item's MMAs read (its blocks' 128 pixels at every tap offset) lies
             // inside the A box that starts at the row of its first pixel
             const int64_t p0 = (int64_t)it.by * 128, y_lo = p0 / s.cols_box;
@@ -1220,14 +1307,30 @@ void pack_weights_bf16(const Net& net, const PlanTables& t, std::vector<uint16_t
     }
 }
 
-void pack_weights_fp32(const Net& net, const PlanTables& t, std::vector<float>& w32,
-                       std::vector<float>& scale, std::vector<float>& bias) {
-    w32.assign((size_t)t.weight32_elems, 0.f);
+void pack_weights_fp32(const Net& net, const PlanTables& t, std::vector<float>& w32) {
+    w32.assign((size_t)t.pack32_elems, 0.f);
+    for (const MafatStageDev& s : t.stages) {
+        const Layer& L = net.layers[s.layer];
+        const std::vector<float>& w = net.w[s.layer];
+        const int taps = L.k * L.k, cc = f32_chunk_channels(L.k);
+        // writes in order; the reads are one stream per output channel of the block
+        for (int nb = 0; nb < s.n_nblk; ++nb) {
+            const int o0 = nb * s.n_blk, n = std::min(s.n_blk, L.c_out - o0);
+            for (int ci = 0; ci < L.c_in; ++ci)
+                for (int tap = 0; tap < taps; ++tap) {
+                    const size_t row = (((size_t)nb * s.f32_chunks + ci / cc) * taps + tap) * cc + ci % cc;
+                    float* dst = w32.data() + s.f32_w_off + row * s.n_blk;
+                    const float* src = w.data() + ((size_t)o0 * L.c_in + ci) * taps + tap;
+                    for (int o = 0; o < n; ++o) dst[o] = src[(size_t)o * L.c_in * taps];
+                }
+        }
+    }
+}
+
+void pack_scale_bias(const Net& net, const PlanTables& t, std::vector<float>& scale, std::vector<float>& bias) {
     scale.assign((size_t)t.sb_elems, 0.f);
     bias.assign((size_t)t.sb_elems, 0.f);
     for (const MafatStageDev& s : t.stages) {
-        const std::vector<float>& w = net.w[s.layer];
-        std::copy(w.begin(), w.end(), w32.begin() + s.w32_off);
         std::copy(net.scale[s.layer].begin(), net.scale[s.layer].end(), scale.begin() + s.sb_off);
         std::copy(net.bias[s.layer].begin(), net.bias[s.layer].end(), bias.begin() + s.sb_off);
     }

@@ -119,6 +119,7 @@ struct PlanTables {
     std::vector<TmapReq> tmaps;          // index i = tensor map i (scratch inputs)
     int64_t weight_elems = 0;            // packed bf16 weight elements
     int64_t weight32_elems = 0;          // fp32 weight elements
+    int64_t pack32_elems = 0;            // fp32 weights as packed for the kernel (with padding)
     int64_t sb_elems = 0;                // scale / bias elements
     int64_t slot_buf_elems = 0;          // elements of one ping-pong buffer
     int64_t scratch_elems = 0;           // the scratch allocation (ring, or layer maps with halo reuse)
@@ -156,8 +157,9 @@ std::string validate_plan(const Net& net, const PlanTables& t);
 // Pack fp32 weights [cout][cin][k][k] of every stage into the bf16 tensor-core
 // blob order (see pack_weights_bf16 in planner.cpp); out has weight_elems entries.
 void pack_weights_bf16(const Net& net, const PlanTables& t, std::vector<uint16_t>& out);
-void pack_weights_fp32(const Net& net, const PlanTables& t, std::vector<float>& w32,
-                       std::vector<float>& scale, std::vector<float>& bias);
+// fp32 plans: the weights in the order the CUDA-core kernel reads them (MafatStageDev::f32_w_off).
+void pack_weights_fp32(const Net& net, const PlanTables& t, std::vector<float>& w32);
+void pack_scale_bias(const Net& net, const PlanTables& t, std::vector<float>& scale, std::vector<float>& bias);
 
 uint16_t f32_to_bf16_rne(float f);
 

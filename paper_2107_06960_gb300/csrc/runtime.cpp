@@ -434,8 +434,8 @@ mafat_status mafat_plan_ex(const mafat_net_t* net, int32_t n_groups, const int32
         return cuda_fail(e, "cudaGetDevice");
     }
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-    // tensor-core kernel: one CTA per SM (shared memory and TMEM); check kernel: 8 small CTAs per SM
-    p->grid = o.max_ctas > 0 ? o.max_ctas : (dt == MAFAT_BF16 ? sms : 8 * sms);
+    // tensor-core kernel: one CTA per SM (shared memory and TMEM); fp32 kernel: as many as an SM holds
+    p->grid = o.max_ctas > 0 ? o.max_ctas : (dt == MAFAT_BF16 ? sms : mafat_fp32_ctas_per_sm() * sms);
     if (p->grid <= 0) p->grid = 1;
 
     auto bail = [&](cudaError_t ee, const char* what) {
@@ -459,8 +459,8 @@ mafat_status mafat_plan_ex(const mafat_net_t* net, int32_t n_groups, const int32
     if (t.cfg.n_groups >= 2 && (e = dalloc(p, &p->d_cut, p->cut_bytes)) != cudaSuccess) return bail(e, "cudaMalloc");
     if (t.in_convert && (e = dalloc(p, &p->d_in_planar, p->in_planar_bytes)) != cudaSuccess) return bail(e, "cudaMalloc");
 
-    std::vector<float> w32, sc, bi;
-    mafat::pack_weights_fp32(net->net, t, w32, sc, bi);
+    std::vector<float> sc, bi;
+    mafat::pack_scale_bias(net->net, t, sc, bi);
     if (dt == MAFAT_BF16) {
         std::vector<uint16_t> wb;
         mafat::pack_weights_bf16(net->net, t, wb);
@@ -468,6 +468,8 @@ mafat_status mafat_plan_ex(const mafat_net_t* net, int32_t n_groups, const int32
         if ((e = cudaMemcpy(p->d_w, wb.data(), wb.size() * 2, cudaMemcpyHostToDevice)) != cudaSuccess)
             return bail(e, "cudaMemcpy");
     } else {
+        std::vector<float> w32;
+        mafat::pack_weights_fp32(net->net, t, w32);
         if ((e = dalloc(p, &p->d_w, w32.size() * 4)) != cudaSuccess) return bail(e, "cudaMalloc");
         if ((e = cudaMemcpy(p->d_w, w32.data(), w32.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess)
             return bail(e, "cudaMemcpy");
@@ -768,7 +770,7 @@ mafat_status mafat_plan_stats(const mafat_plan_t* plan, mafat_plan_stats_t* out)
     s.weight_bytes = plan->weight_bytes;
     s.scratch_bytes = plan->scratch_bytes;
     s.workspace_bytes = plan->workspace_bytes;
-    s.smem_bytes_per_cta = plan->dtype == MAFAT_BF16 ? (int64_t)mafat_tc_smem_bytes() : 4;
+    s.smem_bytes_per_cta = plan->dtype == MAFAT_BF16 ? (int64_t)mafat_tc_smem_bytes() : (int64_t)mafat_fp32_smem_bytes();
     s.ring_slots = t.ring_slots;
     s.wave_tiles = t.wave_tiles;
     s.max_ctas = plan->grid;
