@@ -630,7 +630,19 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                 buf = std::max(buf, (int64_t)r.h() * r.w() * ceil_div(st.cout, 8) * 8);
             }
     t.slot_buf_elems = (buf + 127) / 128 * 128;  // 256-byte aligned for bf16, 512 for fp32
-    t.scratch_elems = (int64_t)S * 2 * t.slot_buf_elems;
+    // Several frames with a ring each, where that stays small, so that a frame's first tiles need
+    // not wait for the last stages of the frame before: a frame's chain of layers is longer than
+    // the time its work keeps the SMs busy.  The limit keeps the rings in the 129 MB L2; an fp32
+    // plan's also leave room in the 32 MiB area of the allocation-free call.
+    const bool reorder = cfg.batch > 1 && !cfg.halo_reuse && !cfg.frame_major && cfg.ring_slots <= 0 && cfg.wave_tiles <= 0 &&
+                         W >= max_tiles && S >= tiles_per_frame;
+    if (reorder && cfg.batch > 1 && S == tiles_per_frame) {
+        const int64_t set_bytes = (int64_t)S * 2 * t.slot_buf_elems * (cfg.dtype == 0 ? 2 : 4);
+        const int64_t limit = cfg.dtype == 0 ? (int64_t)112 << 20 : (int64_t)16 << 20;
+        t.ring_sets = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(cfg.batch, 4), limit / std::max<int64_t>(set_bytes, 1)));
+    }
+    const int S_all = S * t.ring_sets;
+    t.scratch_elems = (int64_t)S_all * 2 * t.slot_buf_elems;
     // halo reuse: one whole output map per non-final stage, every frame, instead of the ring
     std::vector<int64_t> map_off(t.stages.size(), -1), map_frame(t.stages.size(), 0);
     std::vector<int> map_h(t.stages.size(), 0), map_w(t.stages.size(), 0), stage_tmap(t.stages.size(), -1);
@@ -694,11 +706,6 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
     }
 
     // ---- tasks in hand-out order, with their dependencies expressed as task indices
-    struct TaskDep {
-        int prev_task = -1;    // previous stage of the same tile, or the ring predecessor's last stage
-        int group_ctr = -1;    // (frame, group) counter whose group must be complete (first stages)
-        int bump_ctr = -1;     // (frame, group) counter this last stage of a group bumps
-    };
     std::vector<TaskDep> deps;
     std::vector<int> last_task_of_seq;
     int seq = 0;
@@ -720,7 +727,7 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                     for (size_t q = w0; q < w1; ++q) {
                         const TileInfo& ti = tl[q];
                         int tseq = seq + (int)(q - w0);
-                        int slot = tseq % S;
+                        int slot = tseq % S_all;
                         MafatTaskDev tk{};
                         tk.stage = s;
                         tk.frame = f;
@@ -831,7 +838,7 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                         TaskDep d;
                         int qi = (int)(q - w0);
                         if (s == t.stage_first[g]) {
-                            if (!cfg.halo_reuse && tseq >= S) d.prev_task = last_task_of_seq[tseq - S];
+                            if (!cfg.halo_reuse && tseq >= S_all) d.prev_task = last_task_of_seq[tseq - S_all];
                             if (g >= 1) d.group_ctr = f * (G - 1) + (g - 1);
                         } else if (cfg.halo_reuse) {
                             // every previous-stage task whose owned output meets this task's input
@@ -883,12 +890,12 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
     // dependency still points to an earlier task: a first-group task depends on its own frame's
     // earlier tasks and on the same tile of the previous frame (its ring slot); a second-group
     // task on its own frame's first group, all of which was handed out before.
+    std::vector<int> order;
     if (cfg.batch > 1 && G == 2 && !cfg.halo_reuse && !cfg.frame_major && S >= tiles_per_frame && W >= max_tiles) {
         const int n_t = (int)t.tasks.size();
         std::vector<std::vector<int>> fill(cfg.batch), chain(cfg.batch);
         for (int i = 0; i < n_t; ++i)
             (t.tasks[i].stage <= t.stage_last[0] ? fill : chain)[t.tasks[i].frame].push_back(i);
-        std::vector<int> order;
         order.reserve(n_t);
         order.insert(order.end(), fill[0].begin(), fill[0].end());
         for (int f = 0; f < cfg.batch; ++f) {
@@ -933,6 +940,31 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
             while (pos < nx.size()) order.push_back(nx[pos++]);
         }
         if ((int)order.size() != n_t) return "internal: frame interleave lost a task";
+        t.frames_overlapped = 1;
+    }
+    // Stages with many items (all tiles of one frame) keep every CTA busy whatever it holds,
+    // so their CTAs take the next ticket early; stages with about a wave of items or fewer
+    // take it only when the CTA can start it, so that no idle CTA waits for a busy one.
+    // With frames overlapped the next frame keeps every CTA busy in any stage (608x608, 16
+    // frames: 80.4 against 80.9 us per frame).
+    {
+        const int64_t thr = cfg.lookahead_items > 0 ? cfg.lookahead_items
+                            : t.frames_overlapped  ? 1
+                                                   : (int64_t)n_ctas * 5 / 4;
+        std::vector<int64_t> stage_items(t.stages.size(), 0);
+        for (const MafatTaskDev& tk : t.tasks)
+            if (tk.frame == 0) stage_items[tk.stage] += tk.n_items;
+        for (size_t s = 0; s < t.stages.size(); ++s)
+            t.stages[s].lookahead = (cfg.lookahead_items >= 0 && stage_items[s] >= thr) ? 1 : 0;
+    }
+    if (order.empty())
+        for (int i = 0; i < (int)t.tasks.size(); ++i) order.push_back(i);
+    if (reorder) {
+        order = hand_out_order(t, deps, order);
+        if (order.size() != t.tasks.size()) return "internal: the hand-out order lost a task";
+    }
+    {
+        const int n_t = (int)t.tasks.size();
         std::vector<int> new_of(n_t);
         for (int k = 0; k < n_t; ++k) new_of[order[k]] = k;
         std::vector<MafatTaskDev> tasks2(n_t);
@@ -946,7 +978,6 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
         deps.swap(deps2);
         for (TmapReq& r : t.tmaps)
             if (r.task >= 0) r.task = new_of[r.task];
-        t.frames_overlapped = 1;
     }
 
     // ---- counters: one per task, then one per frame (group-1 completion)
@@ -1008,22 +1039,6 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                 }
     }
     if (t.items.size() > (size_t)0x7fffffff) return "too many work items";
-    // Stages with many items (all tiles of one frame) keep every CTA busy whatever it holds,
-    // so their CTAs take the next ticket early; stages with about a wave of items or fewer
-    // take it only when the CTA can start it, so that no idle CTA waits for a busy one.
-    // With frames overlapped the next frame keeps every CTA busy in any stage (608x608, 16
-    // frames: 80.4 against 80.9 us per frame).
-    {
-        const int n_ctas = cfg.n_ctas > 0 ? cfg.n_ctas : 152;
-        const int64_t thr = cfg.lookahead_items > 0 ? cfg.lookahead_items
-                            : t.frames_overlapped  ? 1
-                                                   : (int64_t)n_ctas * 5 / 4;
-        std::vector<int64_t> stage_items(t.stages.size(), 0);
-        for (const MafatTaskDev& tk : t.tasks)
-            if (tk.frame == 0) stage_items[tk.stage] += tk.n_items;
-        for (size_t s = 0; s < t.stages.size(); ++s)
-            t.stages[s].lookahead = (cfg.lookahead_items >= 0 && stage_items[s] >= thr) ? 1 : 0;
-    }
 
     // ---- statistics
     for (int l = 0; l < n; ++l) {
@@ -1053,7 +1068,7 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
     const int64_t cut_total = (int64_t)t.cfg.batch * t.cut_c8 * 8 * t.cut_h * t.cut_w;
     const int64_t out_total = (int64_t)t.cfg.batch * t.out_h * t.out_w * t.out_c;
     const int64_t scratch_total = t.scratch_elems;
-    if (!t.cfg.halo_reuse && scratch_total < (int64_t)t.ring_slots * 2 * t.slot_buf_elems) return "scratch below the ring";
+    if (!t.cfg.halo_reuse && scratch_total < (int64_t)t.ring_slots * t.ring_sets * 2 * t.slot_buf_elems) return "scratch below the ring";
     auto buf_total = [&](int kind) {
         return kind == MAFAT_BUF_USER_IN ? in_total
                : kind == MAFAT_BUF_CUT   ? cut_total
@@ -1265,44 +1280,42 @@ void pack_weights_bf16(const Net& net, const PlanTables& t, std::vector<uint16_t
                 for (int b = 0; b < s.n_bsteps; ++b) {
                     size_t blob = (size_t)s.w_off +
                                   ((size_t)(nb * s.n_chunks + c) * s.n_bsteps + b) * (size_t)s.blob_elems;
+                    const int n = std::min(s.n_blk, L.c_out - nb * s.n_blk);  // the rest is zero padding
                     for (int j = 0; j < s.kst; ++j)
-                        for (int h = 0; h < 2; ++h)
-                            for (int nn = 0; nn < s.n_blk; ++nn)
-                                for (int e = 0; e < 8; ++e) {
-                                    int o = nb * s.n_blk + nn;
-                                    int ci, tap;
-                                    if (s.pix_pair) {
-                                        const int kx = 2 * h + (e >> 2);
-                                        tap = kx < k ? b * k + kx : -1;
-                                        ci = e & 3;
-                                    } else if (s.paired) {
-                                        int a = 2 * b, bb = 2 * b + 1;
-                                        if (bb >= taps) {
-                                            a = -1;  // zero weights paired with the last tap
-                                            bb = taps - 1;
-                                        }
-                                        tap = h == 0 ? a : bb;
-                                        ci = e;
-                                    } else {
-                                        tap = b;
-                                        ci = ((c * s.chunk8) + 2 * j + h) * 8 + e;
+                        for (int h = 0; h < 2; ++h) {
+                            // eight elements (e) of K half h of step j: input channel and tap of
+                            // each, as offsets into an output channel's [cin][taps] (-1: zero)
+                            int from[8];
+                            for (int e = 0; e < 8; ++e) {
+                                int ci, tap;
+                                if (s.pix_pair) {
+                                    const int kx = 2 * h + (e >> 2);
+                                    tap = kx < k ? b * k + kx : -1;
+                                    ci = e & 3;
+                                } else if (s.paired) {
+                                    int a = 2 * b, bb = 2 * b + 1;
+                                    if (bb >= taps) {
+                                        a = -1;  // zero weights paired with the last tap
+                                        bb = taps - 1;
                                     }
-                                    float v = 0.f;
-                                    if (tap >= 0 && ci < cin && o < L.c_out) {
-                                        int ky = tap / k, kx = tap % k;
-                                        v = w[(((size_t)o * cin + ci) * k + ky) * k + kx];
-                                    }
-                                    size_t idx;
-                                    if (s.b_swz) {
-                                        const int u = 2 * j + h;  // 16-byte unit of the 128-byte row
-                                        idx = blob + (size_t)(nn / 8) * 512 + (size_t)(nn % 8) * 64 +
-                                              (size_t)((u ^ (nn % 8)) * 8) + e;
-                                    } else {
-                                        idx = blob + (size_t)j * 2 * s.n_blk * 8 + (size_t)h * s.n_blk * 8 +
-                                              (size_t)(nn / 8) * 64 + (size_t)(nn % 8) * 8 + e;
-                                    }
-                                    out[idx] = f32_to_bf16_rne(v);
+                                    tap = h == 0 ? a : bb;
+                                    ci = e;
+                                } else {
+                                    tap = b;
+                                    ci = ((c * s.chunk8) + 2 * j + h) * 8 + e;
                                 }
+                                from[e] = tap >= 0 && ci < cin ? ci * taps + tap : -1;
+                            }
+                            const float* src = w.data() + (size_t)nb * s.n_blk * cin * taps;
+                            for (int nn = 0; nn < n; ++nn, src += (size_t)cin * taps) {
+                                // swizzled: 16-byte unit 2j + h of the channel's 128-byte row
+                                uint16_t* dst = out.data() + blob +
+                                                (s.b_swz ? (size_t)(nn / 8) * 512 + (size_t)(nn % 8) * 64 +
+                                                               (size_t)(((2 * j + h) ^ (nn % 8)) * 8)
+                                                         : ((size_t)j * 2 + h) * s.n_blk * 8 + (size_t)nn * 8);
+                                for (int e = 0; e < 8; ++e) dst[e] = from[e] >= 0 ? f32_to_bf16_rne(src[from[e]]) : 0;
+                            }
+                        }
                 }
     }
 }

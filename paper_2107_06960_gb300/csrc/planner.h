@@ -125,6 +125,7 @@ struct PlanTables {
     int64_t scratch_elems = 0;           // the scratch allocation (ring, or layer maps with halo reuse)
     std::vector<MafatDepDev> deps;       // task dependency lists (halo reuse)
     int ring_slots = 0, wave_tiles = 0;
+    int ring_sets = 1;                   // rings of ring_slots tiles: consecutive frames take turns
     int n_counters = 0;                  // words after MAFAT_CTR_BASE
     int frame_ctr_base = 0;              // completion counters of every group but the last, per frame:
                                          // frame_ctr_base + frame * (n_groups - 1) + group
@@ -143,6 +144,16 @@ struct PlanTables {
     double useful_flops = 0, executed_flops = 0, issued_flops = 0, predicted_mib = 0;
     int64_t group_io_elems = 0;
 };
+
+// Dependencies of a task, by task index.
+struct TaskDep {
+    int prev_task = -1;    // previous stage of the same tile, or the ring predecessor's last stage
+    int group_ctr = -1;    // (frame, group) counter whose group must be complete (first stages)
+    int bump_ctr = -1;     // (frame, group) counter this last stage of a group bumps
+};
+
+// The order in which the tasks are handed out (indices into t.tasks): `given`, or a better one.
+std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& given);
 
 // Lower a configuration; returns "" or an error message.  `unsupported` is
 // set when the configuration is valid but not implemented.

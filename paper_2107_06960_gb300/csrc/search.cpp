@@ -117,6 +117,20 @@ mafat_status mafat_search_measured(const mafat_net_t* net, const mafat_search_op
         po.dry_run = 1;
         mafat_plan_t* plan = nullptr;
         st = mafat_plan_ex(net, c.n_groups, &cut, c.gn, c.gm, batch, opt->dtype, &po, &plan);
+        mafat_plan_options run_po{};
+        run_po.struct_size = (int32_t)sizeof(run_po);
+        run_po.test_unpublished_task = -1;
+        if (st == MAFAT_OK && batch > 1) {
+            // candidates are compared, and held to the budget, with one ring of tiles: the rings a
+            // batched plan adds where memory is plentiful would count against a budget that it fits
+            mafat_plan_stats_t ps{};
+            ps.struct_size = (int32_t)sizeof(ps);
+            mafat_plan_stats(plan, &ps);
+            mafat_plan_destroy(plan);
+            plan = nullptr;
+            po.ring_slots = run_po.ring_slots = ps.ring_slots;
+            st = mafat_plan_ex(net, c.n_groups, &cut, c.gn, c.gm, batch, opt->dtype, &po, &plan);
+        }
         if (st == MAFAT_OK) {
             mafat_plan_stats_t ps{};
             ps.struct_size = (int32_t)sizeof(ps);
@@ -137,7 +151,7 @@ mafat_status mafat_search_measured(const mafat_net_t* net, const mafat_search_op
             r.status = st;
         }
         if (!dry && r.status == MAFAT_OK) {
-            st = mafat_plan_ex(net, c.n_groups, &cut, c.gn, c.gm, batch, opt->dtype, nullptr, &plan);
+            st = mafat_plan_ex(net, c.n_groups, &cut, c.gn, c.gm, batch, opt->dtype, &run_po, &plan);
             if (st != MAFAT_OK) {
                 r.status = st;
             } else {
