@@ -21,6 +21,7 @@
 // row are adjacent, so 8 pixels x 8 channels form one contiguous 128-byte
 // tensor-core core matrix at any pixel offset.
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 
 #if defined(__CUDACC__)
@@ -35,7 +36,7 @@
 #define MAFAT_MAX_MB_PAIRED 8  // M blocks per work item of a paired-tap (8-input-channel) layer
 #define MAFAT_MAX_NBLK 256  // output channels of one item (MMA N)
 #define MAFAT_A_STAGE_BYTES 36864   // shared-memory A halo stage of the tensor-core kernel (x2)
-#define MAFAT_B_PIECE_BYTES 75776   // one of the two shared-memory weight buffers (x2)
+#define MAFAT_B_PIECE_BYTES 74752   // one of the two shared-memory weight buffers (x2)
 
 // SCRATCH: a tile's own region buffer in the scratch ring (frame in the offset); MAP: a
 // whole layer-output map of every frame in the scratch allocation (halo reuse: tiles
@@ -80,7 +81,8 @@ struct MafatStageDev {
     int32_t bpp;          // blobs per weight piece (a piece fills at most one shared-memory buffer)
     int32_t n_pieces;     // pieces per channel block (1: the set stays resident across items)
     int32_t sb_off;       // offset into the scale / bias arrays
-    int32_t lookahead;    // 1: a CTA takes its next item as soon as this stage's item is loaded
+    int32_t lookahead;    // when a CTA takes its next item: 2 as soon as this stage's item has its inputs,
+                          // 1 once it is loaded, 0 once the next item's first loads could go out
     // fp32 plans (CUDA-core kernel).  A task's conv region is cut into groups of 8 neighbouring
     // pixels of a row, nbx per row: row by row (row pair by row pair, the two rows of a pair
     // alternating, where a pool follows), or in blocks of f32_groups rows x one group column
@@ -186,6 +188,97 @@ struct MafatItemDev {
     int32_t dep1, dep1_target;
     int32_t extra_ctr;    // second counter bumped on completion (-1: none)
 };
+
+// ---------------------------------------------------------------------------
+// Item records of the tensor-core kernel: everything its warps need of an item, built once per
+// plan on the host, so that handing an item out on the device is one 256-byte copy from L2 into
+// a queue slot instead of three dependent table reads and their assembly.  Every role reads only
+// its own part.
+
+// What the epilogue and the publisher need.
+struct MafatEpiRec {
+    int64_t out_off;         // element offset of the task's output in its buffer (frame and tile included)
+    int32_t x0, xlim;        // conv column of the item's block column; end of the task's columns
+    int32_t y0, ylim;        // conv row of the item's first block row; end of the task's rows
+    int32_t out_y0, out_x0;  // map position of output buffer pixel (0, 0)
+    int32_t out_w, out_h;    // output buffer extent (pixels, after pooling)
+    int16_t nbk;             // blocks of the item
+    int16_t nby;             // per-block-halo item: block rows of its task (0: blocks stacked from y0)
+    int32_t n_blk;           // output channels per item (accumulator columns per block)
+    int32_t cout, ch_base;   // channels of the layer; first channel of the item
+    int32_t flags;           // bit 0: fused max-pool, bit 1: NHWC output, bit 2: never published (test
+                             // hook), bits 4-6: MAFAT_BUF_* of the output
+    int32_t done_ctr, extra_ctr;
+    int16_t chain;           // 1: chain item (first pass turns the 3x3's result into the 1x1's A operand)
+    int16_t n_mid;           // chain item: columns of the 3x3's accumulator
+    int16_t a_col, out_col;  // chain item: TMEM columns of the 1x1's A operand and of its accumulator
+    int16_t pitch;           // flat stage: row pitch of the region (pixels); 0: 16x8 blocks
+    int16_t flat_by;         // flat stage: the item's first block in the region; per-block-halo item:
+                             // its first block's index in the task's column-major block order
+};
+
+// What the MMA issuer needs, packed in 32-bit words that it reads with three 16-byte
+// shared-memory loads and broadcasts word by word (the read is on the MMA warp's path between
+// items, while the tensor core keeps shared memory busy with its operands):
+//   w[0] key: stage * 256 + channel block, identifies a resident weight set
+//   w[1] sb: offset of the item's first channel in the scale / bias arrays
+//   w[2] bytes of one weight blob
+//   w[3] n_mid: MMA N of the item's (first) convolution
+//   w[4] k | K steps per blob << 8 | blocks << 16 | paired << 24 | swizzled B << 25 | chain << 26 |
+//        pixel pairs << 27 | per-block halos << 28
+//   w[5] A box columns | rows << 16
+//   w[6] input chunks | blobs per chunk << 16
+//   w[7] blobs per weight piece | pieces << 16
+//   w[8] flat stage: A box pixel of the item's first pixel + 1 (0: 16x8 blocks) | box pixels << 16
+struct MafatMmaRec {
+    uint32_t w[12];
+};
+
+// What the MMA issuer needs of a chain item's chained 1x1 (N, input chunks, K steps per blob,
+// swizzled blobs, blobs per piece, pieces, TMEM columns of its A operand and accumulator,
+// blob elements, scale / bias offset).  Read from the queue slot only on the chain path.
+struct MafatChainRec {
+    int16_t n2, nch2, kst2, swz2, bpp2, np2, a_col, out_col;
+    int32_t blob2, sb2;
+    int64_t w_off2;          // element offset of its packed weights (for the loader)
+};
+
+// What the gather warp needs of an item that reads raw NHWC rows (MAFAT_IN_GATHER).
+struct MafatGatherRec {
+    int16_t on;              // 1: this item's A halo is built from raw rows by the gather warp,
+                             // one pixel per 16-byte slot; 2: two pixels per slot (pixel pairs)
+    int16_t c;               // channels of the input (1..7)
+    int16_t raw_e;           // elements of one raw row in shared memory
+    int16_t s0;              // element of the first halo pixel's channel 0 within a raw row
+};
+
+// What the loader needs: dependencies, the weight set and the A boxes.
+struct MafatLoadRec {
+    int32_t dep0, dep0_target, dep1, dep1_target;  // completion counters to wait for (-1: none)
+    int32_t task, dep_first, dep_count;            // halo reuse: the task's dependency list
+    int32_t map;             // tensor map of the input (-1: the kernel's user-input map)
+    int64_t w_off;           // element offset of the item's packed weight set
+    int32_t x0, y0;          // box position: elements along x (gather: pixel columns) and row
+    int32_t c3;              // frame coordinate
+    int32_t a_bytes;         // bytes of one A box
+    int16_t chunk8;          // input octets per chunk (third coordinate step)
+    int16_t lookahead;       // MafatStageDev::lookahead
+    int16_t g_nby, g_by;     // gather item: block rows of its task, first block of the item
+    int16_t g_pad, g_k;      // gather item: reserved, kernel size
+    int32_t g_cin;           // gather item: channels of the image
+};
+
+struct alignas(16) MafatItemRec {
+    MafatEpiRec epi;         // 80 bytes
+    MafatMmaRec mma;         // 48
+    MafatChainRec chain;     // 32
+    MafatGatherRec gather;   // 8
+    MafatLoadRec load;       // 72
+    int32_t reserved[4];
+};
+#define MAFAT_REC_BYTES 256
+static_assert(sizeof(MafatItemRec) == MAFAT_REC_BYTES, "item record");
+static_assert(offsetof(MafatItemRec, mma) % 16 == 0, "16-byte loads of the MMA record");
 
 // Counter block layout (uint32 words).  Zeroed when the plan is created; the
 // last CTA to leave a run sets every word except the status back to zero, so

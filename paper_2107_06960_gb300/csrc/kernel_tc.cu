@@ -28,15 +28,16 @@
 //    it, larger sets stream piece by piece (every copy costs a few hundred cycles
 //    of TMA time however small it is, so copies are large and few).
 //
-// Warp roles (384 threads): warps 0-7 epilogue (warp w reads TMEM lanes
+// Warp roles (416 threads): warps 0-7 epilogue (warp w reads TMEM lanes
 // 32(w%4)..+31 = conv rows 4(w%4)..+3 of a block; the two warpgroups take units
-// of one block x 32 columns in turn), warp 8 scheduler + TMA producer, warp 9 TMEM
+// of one block x 32 columns in turn), warp 8 loader (dependencies, TMA), warp 9 TMEM
 // allocator + MMA issuer, warp 10 publisher (bumps an item's completion counter
 // once all epilogue threads have stored it, so that the epilogue warps never wait
 // for their stores to reach L2), warp 11 gather (expands raw rows of a narrow NHWC
-// input image, e.g. 3-channel RGB, into the 8-channel halo layout of the first layer).  Shared memory: 2 A halo stages, 2 weight
-// buffers, a 4-deep queue of items with the record the epilogue needs (written by
-// the producer, so the epilogue reads no work table from global memory), and one
+// input image, e.g. 3-channel RGB, into the 8-channel halo layout of the first layer), warp 12
+// scheduler (tickets and item records).  Shared memory: 2 A halo stages, 2 weight
+// buffers, a 4-deep queue of item records (copied in by the scheduler, so no other role
+// reads a work table from global memory), and one
 // scale / bias slot per accumulator (copied in by the MMA warp and landing on the
 // accumulator's full barrier); TMEM: 2 accumulators of 256 columns (the epilogue
 // of one item overlaps the MMAs of the next).
@@ -59,7 +60,8 @@ constexpr int kProducerWarp = kEpiWarps;
 constexpr int kMmaWarp = kEpiWarps + 1;
 constexpr int kPubWarp = kEpiWarps + 2;
 constexpr int kGatherWarp = kEpiWarps + 3;
-constexpr int kThreads = (kEpiWarps + 4) * 32;
+constexpr int kSchedWarp = kEpiWarps + 4;
+constexpr int kThreads = (kEpiWarps + 5) * 32;
 constexpr int kAStages = 2;
 constexpr int kQDepth = 4;
 constexpr int kAStageBytes = MAFAT_A_STAGE_BYTES;   // one A halo box, multiple of 1024
@@ -81,13 +83,14 @@ constexpr int kBarEpiDone = kBarDone + 1;          // every epilogue thread has 
 constexpr int kBarPubDone = kBarEpiDone + 2;       // the publisher has published item e (slot e % 2)
 constexpr int kBarRawFull = kBarPubDone + 2;       // raw NHWC rows have landed in A stage s (gather items)
 constexpr int kBarMidFull = kBarRawFull + kAStages; // chain items: the 3x3's bf16 result is in TMEM (buffer b)
-constexpr int kNumBars = kBarMidFull + 2;
-constexpr int kOffRec = 256;                        // kQDepth epilogue records
-constexpr int kRecStride = 160;
+constexpr int kBarTake = kBarMidFull + 2;          // the scheduler may take the next ticket
+constexpr int kNumBars = kBarTake + 1;
+constexpr int kOffRec = 256;                        // kQDepth item records
+constexpr int kRecStride = MAFAT_REC_BYTES;
 constexpr int kOffQItems = kOffRec + kQDepth * kRecStride;
 constexpr int kOffTmem = kOffQItems + 4 * kQDepth;
 constexpr int kOffBroken = kOffTmem + 4;
-constexpr int kOffA = 1024;
+constexpr int kOffA = 2048;
 constexpr int kOffB = kOffA + kAStages * kAStageBytes;
 constexpr int kSbSlotBytes = 2 * MAFAT_MAX_NBLK * 4;  // scale then bias of one item's channels
 constexpr int kOffSb = kOffB + 2 * kBPieceBytes;
@@ -442,73 +445,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
         : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
-
-// What the MMA issuer needs of an item, packed in 32-bit words that it reads with three
-// 16-byte shared-memory loads and broadcasts word by word (the read is on the MMA warp's
-// path between items, while the tensor core keeps shared memory busy with its operands):
-//   w[0] key: stage * 256 + channel block, identifies a resident weight set
-//   w[1] sb: offset of the item's first channel in the scale / bias arrays
-//   w[2] bytes of one weight blob
-//   w[3] n_mid: MMA N of the item's (first) convolution
-//   w[4] k | K steps per blob << 8 | blocks << 16 | paired << 24 | swizzled B << 25 | chain << 26 |
-//        pixel pairs << 27 | per-block halos << 28
-//   w[5] A box columns | rows << 16
-//   w[6] input chunks | blobs per chunk << 16
-//   w[7] blobs per weight piece | pieces << 16
-//   w[8] flat stage: A box pixel of the item's first pixel + 1 (0: 16x8 blocks) | box pixels << 16
-struct __align__(16) MmaRec {
-    uint32_t w[12];
-};
-
-// What the MMA issuer needs of a chain item's chained 1x1 (N, input chunks, K steps per blob,
-// swizzled blobs, blobs per piece, pieces, TMEM columns of its A operand and accumulator,
-// blob elements, scale / bias offset).  Read from the queue slot only on the chain path.
-struct __align__(8) ChainRec {
-    int16_t n2, nch2, kst2, swz2, bpp2, np2, a_col, out_col;
-    int32_t blob2, sb2;
-};
-
-// What the MMA issuer, the epilogue and the publisher need of an item, written into its
-// queue slot by the producer (which has the work tables in registers anyway), so that
-// none of them reads a work table from global memory on its critical path.
-// What the gather warp needs of an item that reads raw NHWC rows (MAFAT_IN_GATHER).
-struct __align__(8) GatherRec {
-    int16_t on;              // 1: this item's A halo is built from raw rows by the gather warp,
-                             // one pixel per 16-byte slot; 2: two pixels per slot (pixel pairs)
-    int16_t c;               // channels of the input (1..7)
-    int16_t raw_e;           // elements of one raw row in shared memory
-    int16_t s0;              // element of the first halo pixel's channel 0 within a raw row
-};
-
-struct __align__(16) EpiRec {  // 16-byte aligned: written and read with 16-byte accesses
-    __nv_bfloat16* out;      // output buffer of the task (frame and tile offset applied)
-    int32_t x0, xlim;        // conv column of the item's block column; end of the task's columns
-    int32_t y0, ylim;        // conv row of the item's first block row; end of the task's rows
-    int32_t out_y0, out_x0;  // map position of output buffer pixel (0, 0)
-    int32_t out_w, out_h;    // output buffer extent (pixels, after pooling)
-    int16_t nbk;             // blocks of the item
-    int16_t nby;             // per-block-halo item: block rows of its task (0: blocks stacked from y0)
-    int32_t n_blk;           // output channels per item (accumulator columns per block)
-    int32_t cout, ch_base;   // channels of the layer; first channel of the item
-    int32_t flags;           // bit 0: fused max-pool, bit 1: NHWC output, bit 2: never published (test hook)
-    int32_t done_ctr, extra_ctr;
-    int16_t chain;           // 1: chain item (first pass turns the 3x3's result into the 1x1's A operand)
-    int16_t n_mid;           // chain item: columns of the 3x3's accumulator
-    int16_t a_col, out_col;  // chain item: TMEM columns of the 1x1's A operand and of its accumulator
-    int16_t pitch;           // flat stage: row pitch of the region (pixels); 0: 16x8 blocks
-    int16_t flat_by;         // flat stage: the item's first block in the region; per-block-halo item:
-                             // its first block's index in the task's column-major block order
-};
-
-// A queue slot: the record of one item, in parts, so that every role copies only its own.
-struct ItemRec {
-    EpiRec epi;
-    MmaRec mma;
-    ChainRec chain;
-    GatherRec gather;
-};
-static_assert(sizeof(ItemRec) <= kRecStride, "item record");
-static_assert(kRecStride % 16 == 0 && offsetof(ItemRec, mma) % 16 == 0, "16-byte loads of the MMA record");
 
 // Where one thread's epilogue results go: its pixel's element offset in the
 // output buffer (octet-planar: offset inside an 8-channel plane; NHWC: offset
@@ -1016,16 +952,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile int* q_items = reinterpret_cast<volatile int*>(smem + kOffQItems);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kOffTmem);
     volatile int* broken = reinterpret_cast<volatile int*>(smem + kOffBroken);
-    ItemRec* recs = reinterpret_cast<ItemRec*>(smem + kOffRec);
+    MafatItemRec* recs = reinterpret_cast<MafatItemRec*>(smem + kOffRec);
     auto bar = [&](int i) { return sbase + (uint32_t)(i * 8); };
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int64_t pipe_limit = 4 * p.timeout_ns + 1000000000LL;
     unsigned long long* const trace = kTrace ? p.trace : nullptr;
-    // the producer's first item record, in flight while the CTA sets up
-    MafatItemDev it_first{};
-    if (warp == kProducerWarp && lane == 0 && (int)blockIdx.x < p.n_items) it_first = p.items[blockIdx.x];
+    // the scheduler's first item record, in flight while the CTA sets up
+    uint4 rec_first = make_uint4(0u, 0u, 0u, 0u);
+    if (warp == kSchedWarp && lane < MAFAT_REC_BYTES / 16 && (int)blockIdx.x < p.n_items)
+        rec_first = __ldg(reinterpret_cast<const uint4*>(p.recs + blockIdx.x) + lane);
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kAStages; ++i) {
@@ -1042,11 +979,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int i = 0; i < kQDepth; ++i) {
             mbar_init(bar(kBarQFull + i), 1);
-            mbar_init(bar(kBarQEmpty + i), kEpiWarps + 3);  // epilogue warps, MMA warp, publisher, gather warp
+            mbar_init(bar(kBarQEmpty + i), kEpiWarps + 4);  // epilogue warps, MMA warp, publisher, gather warp, loader
         }
         for (int i = 0; i < kAStages; ++i) mbar_init(bar(kBarRawFull + i), 1);
         for (int i = 0; i < 2; ++i) mbar_init(bar(kBarMidFull + i), kEpiThreads);
         mbar_init(bar(kBarDone), 1);
+        mbar_init(bar(kBarTake), 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(kBarEpiDone + i), kEpiThreads);
             mbar_init(bar(kBarPubDone + i), 1);
@@ -1067,144 +1005,85 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    if (warp == kProducerWarp) {
-        // ------------------------------------------------------------ scheduler + TMA producer
+    if (warp == kSchedWarp) {
+        // ------------------------------------------------------------ scheduler (warp 12)
+        // Takes tickets and copies each item's record into its queue slot (16 lanes, 16 bytes
+        // each).  The first ticket is the CTA's index (the first gridDim.x items go out at once
+        // anyway); later ones come from the atomic counter, offset by gridDim.x.  When the next
+        // one may be taken is the loader's to say (kBarTake, MafatLoadRec::lookahead): with frames
+        // in flight, once the inputs of its current item are ready; else once the item's loads
+        // are out, or, after an item of a stage with few items, once the A stage the new item
+        // will use is about to free, so that a CTA busy with a long item does not hold work
+        // another CTA could start now (608x608: one frame 93.1 us taking it after the loads, 94.4
+        // before them; 16 frames 876 and 820).  The ticket atomic and the record load (~0.7 us each from
+        // L2) then overlap the loader's work and the current MMAs: with one thread doing both
+        // jobs in turn, three dependent table reads and the record's assembly included, a CTA
+        // started an item every ~2.6 us whatever its MMAs took.
+        uint32_t q_cnt = 0;
+        int ticket = (int)blockIdx.x < p.n_items ? (int)blockIdx.x : -1;
+        uint4 rec = rec_first;
+        while (true) {
+            const int qs = (int)(q_cnt % kQDepth);
+            mbar_wait(bar(kBarQEmpty + qs), ((q_cnt / kQDepth) & 1u) ^ 1u, p.ctr, pipe_limit, broken, 64);
+            if (ticket >= 0 && lane < MAFAT_REC_BYTES / 16)
+                reinterpret_cast<uint4*>(smem + kOffRec + qs * kRecStride)[lane] = rec;
+            if (lane == 0) {
+                q_items[qs] = ticket;
+                if (ticket >= 0 && trace) {
+                    mafat_dev::trace_put(trace, ticket, 0, mafat_dev::globaltimer_ns());
+                    mafat_dev::trace_put(trace, ticket, 4, mafat_dev::smid());
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kBarQFull + qs));  // release: the record is visible to the consumers
+            ++q_cnt;
+            if (ticket < 0) break;
+            mbar_wait(bar(kBarTake), (q_cnt - 1u) & 1u, p.ctr, pipe_limit, broken, 32);
+            int next = 0;
+            if (lane == 0) next = (int)(atomicAdd(&p.ctr[MAFAT_CTR_TICKET], 1u) + gridDim.x);
+            next = __shfl_sync(0xffffffffu, next, 0);
+            ticket = next < p.n_items ? next : -1;
+            if (ticket >= 0 && lane < MAFAT_REC_BYTES / 16)
+                rec = __ldg(reinterpret_cast<const uint4*>(p.recs + ticket) + lane);
+        }
+        __syncwarp();
+    } else if (warp == kProducerWarp) {
+        // ------------------------------------------------------------ loader: dependencies, TMA
         if (lane == 0) {
-            // The input, the weights, the work tables and scale / bias are read from DRAM
-            // once per run, mostly by loads that wait for them (the first layer's halos, the
-            // first use of every weight set and table entry on each SM); fetching them into
-            // L2 at once, spread over all CTAs, overlaps those DRAM latencies instead of
-            // paying them item by item.
-            for (int r = 0; r < MAFAT_PF_REGIONS; ++r) prefetch_l2_share(p.pf_ptr[r], p.pf_bytes[r], p.pf_per[r]);
             uint32_t a_cnt = 0, q_cnt = 0;
             WeightBufs wb;
             // dependency counters already seen at (or above) a target: items of one task
             // usually follow each other, so most items skip the round trip to L2
             int ok_idx0 = -1, ok_idx1 = -1, ok_tgt0 = 0, ok_tgt1 = 0;
             int ok_task = -1;  // the last task whose dependency list was found complete
-            // A ticket is taken (and its item record loaded) at the end of the previous item,
-            // once the A stage the new item will use is about to free: early enough to hide
-            // the new item's loads behind the current MMAs, late enough that a CTA busy with a
-            // long item does not hold work another CTA could start now.  After an item of a
-            // stage with many items (lookahead) it is taken at once: every CTA has work then,
-            // and the hand-out latency (atomic, record loads) is hidden behind the A stage's
-            // release instead of added to it.
-            // The first ticket is the CTA's index (the first gridDim.x items go out at once
-            // anyway), its record loaded during the setup; later tickets come from the atomic
-            // counter, offset by gridDim.x.
-            int next = (int)blockIdx.x;
-            MafatItemDev it_next = it_first;
             while (true) {
-                const int ticket = next < p.n_items ? next : -1;
-                const MafatItemDev it = it_next;
-                if (ticket >= 0 && trace) {
-                    mafat_dev::trace_put(trace, ticket, 0, mafat_dev::globaltimer_ns());
-                    mafat_dev::trace_put(trace, ticket, 4, mafat_dev::smid());
-                }
-                MafatTaskDev tk;
-                MafatStageDev st;
-                if (ticket >= 0) {  // two independent loads (the item names its stage)
-                    tk = p.tasks[it.task];
-                    st = p.stages[it.stage];
-                }
-                // a flat stage's item starts at pixel 128 by of its region read row by row: its A box
-                // starts at that pixel's row, the pixel being flat_off pixels into the box
-                int y_lo = 0, flat_off = -1;
-                if (ticket >= 0 && st.flat) {
-                    const int p0 = it.by * 128;
-                    y_lo = p0 / st.cols_box;
-                    flat_off = p0 - y_lo * st.cols_box;
-                }
                 const int qs = (int)(q_cnt % kQDepth);
-                mbar_wait(bar(kBarQEmpty + qs), ((q_cnt / kQDepth) & 1u) ^ 1u, p.ctr, pipe_limit, broken, 64);
-                q_items[qs] = ticket;
-                if (ticket >= 0) {
-                    // the records are built in registers and stored whole (a few wide stores rather
-                    // than one per field, on this single thread while the tensor core keeps the
-                    // shared memory busy)
-                    EpiRec rc{};
-                    MmaRec& rm = recs[qs].mma;
-                    GatherRec rg{};
-                    rc.out = (__nv_bfloat16*)(tk.out_kind == MAFAT_BUF_USER_OUT ? p.user_out
-                                              : tk.out_kind == MAFAT_BUF_CUT    ? p.cut
-                                                                                : p.scratch) +
-                             tk.out_off;
-                    rc.x0 = tk.cx0 + it.bx * MAFAT_BLK_COLS;
-                    rc.xlim = tk.cx0 + tk.cw;
-                    rc.y0 = (flat_off >= 0 || st.blk_halo) ? tk.cy0 : tk.cy0 + it.by * MAFAT_BLK_ROWS;
-                    rc.nby = (int16_t)(st.blk_halo ? tk.nby : 0);
-                    rc.pitch = (int16_t)(flat_off >= 0 ? st.cols_box : 0);
-                    rc.flat_by = it.by;
-                    rc.ylim = tk.cy0 + tk.ch;
-                    rc.out_y0 = tk.out_y0;
-                    rc.out_x0 = tk.out_x0;
-                    rc.out_w = tk.out_w;
-                    rc.out_h = tk.out_h;
-                    rc.nbk = (int16_t)it.nbk;
-                    // what the epilogue stores: the item's own output, or a chain item's 1x1 output
-                    const bool chain = kChain && st.chain;
-                    rc.n_blk = chain ? st.c2_n_blk : st.n_blk;
-                    rc.cout = chain ? st.c2_cout : st.cout;
-                    rc.ch_base = chain ? 0 : it.nb * st.n_blk;
-                    rc.flags = ((chain ? st.c2_pool : st.pool) ? 1 : 0) | (tk.out_nhwc ? 2 : 0) | ((it.flags & 1) ? 4 : 0);
-                    rc.done_ctr = tk.done_ctr;
-                    rc.extra_ctr = it.extra_ctr;
-                    {
-                        uint4* w = reinterpret_cast<uint4*>(rm.w);
-                        w[0] = make_uint4((uint32_t)(tk.stage * 256 + it.nb), (uint32_t)(st.sb_off + it.nb * st.n_blk),
-                                          (uint32_t)(st.blob_elems * 2), (uint32_t)st.n_blk);
-                        w[1] = make_uint4((uint32_t)st.k | ((uint32_t)st.kst << 8) | ((uint32_t)it.nbk << 16) |
-                                              ((uint32_t)st.paired << 24) | ((uint32_t)st.b_swz << 25) |
-                                              ((uint32_t)chain << 26) | ((uint32_t)st.pix_pair << 27) |
-                                              ((uint32_t)st.blk_halo << 28),
-                                          (uint32_t)st.cols_box | ((uint32_t)st.rows_box << 16),
-                                          (uint32_t)st.n_chunks | ((uint32_t)st.n_bsteps << 16),
-                                          (uint32_t)st.bpp | ((uint32_t)st.n_pieces << 16));
-                        w[2] = make_uint4((uint32_t)(flat_off + 1) | ((uint32_t)(st.rows_box * st.cols_box) << 16), 0u, 0u,
-                                          0u);
-                    }
-                    rc.n_mid = (int16_t)st.n_blk;
-                    rc.chain = (int16_t)chain;
-                    if (chain) {
-                        ChainRec rh{};
-                        rh.n2 = (int16_t)st.c2_n_blk;
-                        rh.nch2 = (int16_t)st.c2_n_chunks;
-                        rh.kst2 = (int16_t)st.c2_kst;
-                        rh.swz2 = (int16_t)st.c2_b_swz;
-                        rh.bpp2 = (int16_t)st.c2_bpp;
-                        rh.np2 = (int16_t)st.c2_n_pieces;
-                        rh.a_col = (int16_t)st.chain_a_col;
-                        rh.out_col = (int16_t)st.chain_out_col;
-                        rh.blob2 = st.c2_blob_elems;
-                        rh.sb2 = st.c2_sb_off;
-                        recs[qs].chain = rh;
-                        rc.a_col = (int16_t)st.chain_a_col;
-                        rc.out_col = (int16_t)st.chain_out_col;
-                    }
-                    rg.on = 0;
-                    if (tk.in_kind == MAFAT_BUF_USER_IN && st.in_mode == MAFAT_IN_GATHER) {
-                        const int e_start = (tk.cx0 + it.bx * MAFAT_BLK_COLS - st.pad - tk.in_x0) * st.cin;
-                        rg.on = (int16_t)(st.pix_pair ? 2 : 1);
-                        rg.c = (int16_t)st.cin;
-                        rg.raw_e = (int16_t)st.raw_e;
-                        rg.s0 = (int16_t)(e_start - (e_start & ~7));
-                    }
-                    recs[qs].epi = rc;
-                    recs[qs].gather = rg;
-                }
-                mbar_arrive(bar(kBarQFull + qs));  // release: the record is visible to the consumers
-                ++q_cnt;
+                mbar_wait(bar(kBarQFull + qs), (q_cnt / kQDepth) & 1u, p.ctr, pipe_limit, broken);
+                const int ticket = q_items[qs];
                 if (ticket < 0) break;
+                const MafatLoadRec ld = recs[qs].load;
+                const uint4 w03 = *reinterpret_cast<const uint4*>(recs[qs].mma.w);
+                const uint4 w47 = *reinterpret_cast<const uint4*>(recs[qs].mma.w + 4);
+                const bool chain = kChain && ((w47.x >> 26) & 1u) != 0;
+                const int nbk = (int)((w47.x >> 16) & 0xFFu);
+                const int rows_box = (int)(w47.y >> 16), cols_box = (int)(w47.y & 0xFFFFu);
+                const int n_chunks = (int)(w47.z & 0xFFFFu), n_bsteps = (int)(w47.z >> 16);
+                const int bpp = (int)(w47.w & 0xFFFFu), P = (int)(w47.w >> 16);
+                const int gather_e = recs[qs].gather.on ? (int)recs[qs].gather.raw_e : 0;
+                const MafatChainRec ch = kChain ? recs[qs].chain : MafatChainRec{};
+                mbar_arrive(bar(kBarQEmpty + qs));
+                ++q_cnt;
+                if (*broken) {  // a pipeline wait ran out: records can no longer be trusted, load nothing
+                    mbar_arrive(bar(kBarTake));
+                    continue;
+                }
                 // the tensor map of the item's input (a table in global memory, cold after the
                 // launch) into the TMA unit's descriptor cache while the item waits for its inputs
-                if (tk.in_kind != MAFAT_BUF_USER_IN) {
-                    const CUtensorMap* pm = tk.in_kind == MAFAT_BUF_CUT ? p.tmaps + p.cut_tmap : p.tmaps + tk.in_tmap;
-                    asm volatile("prefetch.tensormap [%0];" ::"l"(pm) : "memory");
-                }
-                const int key = tk.stage * 256 + it.nb;
-                const int P = st.n_pieces, G = st.n_chunks * st.n_bsteps;
-                const uint32_t blob_bytes = (uint32_t)(st.blob_elems * 2);
-                const uint16_t* wset = p.w_bf16 + st.w_off + (size_t)it.nb * (size_t)(st.set_bytes / 2);
+                const CUtensorMap* map = ld.map < 0 ? &in_map : p.tmaps + ld.map;
+                if (ld.map >= 0) asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+                const int key = (int)w03.x, G = n_chunks * n_bsteps;
+                const uint32_t blob_bytes = w03.z;
+                const uint8_t* wset = reinterpret_cast<const uint8_t*>(p.w_bf16 + ld.w_off);
                 const bool resident = P == 1 && wb.resident(key) >= 0;
                 // Loads go out in the order the MMA issuer consumes them: piece 0, then for
                 // every chunk its A halo and the pieces that start inside it.  A piece goes
@@ -1214,105 +1093,95 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int b_ = wb.next;                                                                               \
         wb.next ^= 1;                                                                                         \
         mbar_wait(bar(kBarBEmpty + b_), (wb.loads(b_) & 1u) ^ 1u, p.ctr, pipe_limit, broken, 64);             \
-        const int nblob_ = min(st.bpp, G - (pc) * st.bpp);                                                    \
+        const int nblob_ = min(bpp, G - (pc) * bpp);                                                          \
         const uint32_t bytes_ = (uint32_t)nblob_ * blob_bytes;                                                \
         mbar_arrive_expect_tx(bar(kBarBFull + b_), bytes_);                                                   \
-        bulk_load(sbase + kOffB + b_ * kBPieceBytes, wset + (size_t)(pc) * st.bpp * st.blob_elems, bytes_,    \
+        bulk_load(sbase + kOffB + b_ * kBPieceBytes, wset + (size_t)(pc) * bpp * blob_bytes, bytes_,          \
                   bar(kBarBFull + b_));                                                                        \
         wb.set_loaded(b_, P == 1 ? key : -1, false);                                                          \
     } while (0)
                 if (!resident) MAFAT_LOAD_PIECE(0);  // weights do not depend on other tiles: fetch first
-                const CUtensorMap* map = tk.in_kind == MAFAT_BUF_USER_IN ? &in_map
-                                         : tk.in_kind == MAFAT_BUF_CUT   ? p.tmaps + p.cut_tmap
-                                                                         : p.tmaps + tk.in_tmap;
-                const int c3 = tk.in_kind == MAFAT_BUF_SCRATCH ? 0 : tk.frame;
-                const int in_mode = tk.in_kind == MAFAT_BUF_USER_IN ? st.in_mode : MAFAT_IN_PLANAR;
-                const int px0 = tk.cx0 + it.bx * MAFAT_BLK_COLS - st.pad - tk.in_x0;  // first halo column
-                const int x0 = px0 * 8;
-                const int y0 = tk.cy0 + (flat_off >= 0 ? y_lo : it.by * MAFAT_BLK_ROWS) - st.pad - tk.in_y0;
-                const uint32_t a_bytes = (uint32_t)(st.chunk8 * st.rows_box * st.cols_box * 16);
                 bool waited = false;
-                if (it.dep0 >= 0 && !(it.dep0 == ok_idx0 && it.dep0_target <= ok_tgt0)) {
-                    mafat_dev::wait_counter(p.ctr, it.dep0, it.dep0_target, p.timeout_ns);
-                    ok_idx0 = it.dep0;
-                    ok_tgt0 = it.dep0_target;
+                if (ld.dep0 >= 0 && !(ld.dep0 == ok_idx0 && ld.dep0_target <= ok_tgt0)) {
+                    mafat_dev::wait_counter(p.ctr, ld.dep0, ld.dep0_target, p.timeout_ns);
+                    ok_idx0 = ld.dep0;
+                    ok_tgt0 = ld.dep0_target;
                     waited = true;
                 }
-                if (it.dep1 >= 0 && !(it.dep1 == ok_idx1 && it.dep1_target <= ok_tgt1)) {
-                    mafat_dev::wait_counter(p.ctr, it.dep1, it.dep1_target, p.timeout_ns);
-                    ok_idx1 = it.dep1;
-                    ok_tgt1 = it.dep1_target;
+                if (ld.dep1 >= 0 && !(ld.dep1 == ok_idx1 && ld.dep1_target <= ok_tgt1)) {
+                    mafat_dev::wait_counter(p.ctr, ld.dep1, ld.dep1_target, p.timeout_ns);
+                    ok_idx1 = ld.dep1;
+                    ok_tgt1 = ld.dep1_target;
                     waited = true;
                 }
-                if (tk.dep_count > 0 && it.task != ok_task) {
-                    mafat_dev::wait_dep_list(p.ctr, p.deps, tk.dep_first, tk.dep_count, p.timeout_ns);
-                    ok_task = it.task;
+                if (ld.dep_count > 0 && ld.task != ok_task) {
+                    mafat_dev::wait_dep_list(p.ctr, p.deps, ld.dep_first, ld.dep_count, p.timeout_ns);
+                    ok_task = ld.task;
                     waited = true;
                 }
                 if (waited) mafat_dev::fence_proxy_async_global();
                 if (trace) mafat_dev::trace_put(trace, ticket, 1, mafat_dev::globaltimer_ns());
+                if (ld.lookahead == 2) mbar_arrive(bar(kBarTake));
                 int next_pc = 1;  // the next weight piece to load (piece 0 went first)
-                for (int c = 0; c < st.n_chunks; ++c) {
+                for (int c = 0; c < n_chunks; ++c) {
                     const int as = (int)(a_cnt % kAStages);
                     const uint32_t a_dst = sbase + kOffA + as * kAStageBytes;
                     mbar_wait(bar(kBarAEmpty + as), ((a_cnt / kAStages) & 1u) ^ 1u, p.ctr, pipe_limit, broken, 64);
-                    if (in_mode == MAFAT_IN_GATHER) {
+                    if (gather_e > 0) {
                         // raw NHWC rows of each block's halo, from the 16-byte aligned element at
                         // or before the halo's first one, into the stage's tail block after block;
                         // the gather warp builds the halos from them and completes the stage's
                         // full barrier itself.  The item's blocks run down its task's block
-                        // columns (column-major order from block it.by).
-                        const int hr = MAFAT_BLK_ROWS + st.k - 1;
-                        const uint32_t stride = (uint32_t)mafat_raw_blk_stride(st.k, st.raw_e);
-                        uint32_t dst = a_dst + (uint32_t)mafat_raw_offset(st.rows_box, st.cols_box);
-                        mbar_arrive_expect_tx(bar(kBarRawFull + as), (uint32_t)(it.nbk * hr * st.raw_e * 2));
-                        int bxx = it.by / tk.nby, byy = it.by - bxx * tk.nby;
-                        for (int j = 0; j < it.nbk; ++j, dst += stride) {
-                            const int e = (tk.cx0 + bxx * MAFAT_BLK_COLS - st.pad - tk.in_x0) * st.cin;
-                            tma_load_3d(dst, map, e & ~7, tk.cy0 + byy * MAFAT_BLK_ROWS - st.pad - tk.in_y0, c3,
-                                        bar(kBarRawFull + as));
-                            if (++byy == tk.nby) {
+                        // columns (column-major order from block g_by).
+                        const int hr = MAFAT_BLK_ROWS + ld.g_k - 1;
+                        const uint32_t stride = (uint32_t)mafat_raw_blk_stride(ld.g_k, gather_e);
+                        uint32_t dst = a_dst + (uint32_t)mafat_raw_offset(rows_box, cols_box);
+                        mbar_arrive_expect_tx(bar(kBarRawFull + as), (uint32_t)(nbk * hr * gather_e * 2));
+                        int bxx = ld.g_by / ld.g_nby, byy = ld.g_by - bxx * ld.g_nby;
+                        for (int j = 0; j < nbk; ++j, dst += stride) {
+                            const int e = (ld.x0 + bxx * MAFAT_BLK_COLS) * ld.g_cin;
+                            tma_load_3d(dst, map, e & ~7, ld.y0 + byy * MAFAT_BLK_ROWS, ld.c3, bar(kBarRawFull + as));
+                            if (++byy == ld.g_nby) {
                                 byy = 0;
                                 ++bxx;
                             }
                         }
                     } else {
-                        mbar_arrive_expect_tx(bar(kBarAFull + as), a_bytes);
-                        tma_load_4d(a_dst, map, x0, y0, c * st.chunk8, c3, bar(kBarAFull + as));
+                        mbar_arrive_expect_tx(bar(kBarAFull + as), (uint32_t)ld.a_bytes);
+                        tma_load_4d(a_dst, map, ld.x0, ld.y0, c * ld.chunk8, ld.c3, bar(kBarAFull + as));
                     }
                     ++a_cnt;
                     // the pieces that start inside this chunk (piece pc starts at blob pc * bpp);
                     // no division: on this single thread, a runtime modulo per blob cost ~1.5 us
                     // per chunk of a 3x3 256->512 item
-                    while (next_pc < P && next_pc * st.bpp < (c + 1) * st.n_bsteps) {
+                    while (next_pc < P && next_pc * bpp < (c + 1) * n_bsteps) {
                         MAFAT_LOAD_PIECE(next_pc);
                         ++next_pc;
                     }
                 }
 #undef MAFAT_LOAD_PIECE
-                if (kChain && st.chain) {
+                if (kChain && chain) {
                     // the chained 1x1's weights follow the 3x3's, streamed piece by piece (never
                     // resident), in the order the MMA issuer consumes them
-                    const uint16_t* wset2 = p.w_bf16 + st.c2_w_off;
-                    const int G2 = st.c2_n_chunks;  // one tap per blob
-                    const uint32_t blob_bytes2 = (uint32_t)(st.c2_blob_elems * 2);
-                    for (int pc = 0; pc < st.c2_n_pieces; ++pc) {
+                    const uint16_t* wset2 = p.w_bf16 + ch.w_off2;
+                    const int G2 = ch.nch2;  // one tap per blob
+                    const uint32_t blob_bytes2 = (uint32_t)(ch.blob2 * 2);
+                    for (int pc = 0; pc < ch.np2; ++pc) {
                         const int b_ = wb.next;
                         wb.next ^= 1;
                         mbar_wait(bar(kBarBEmpty + b_), (wb.loads(b_) & 1u) ^ 1u, p.ctr, pipe_limit, broken, 64);
-                        const int nblob_ = min(st.c2_bpp, G2 - pc * st.c2_bpp);
+                        const int nblob_ = min((int)ch.bpp2, G2 - pc * ch.bpp2);
                         const uint32_t bytes_ = (uint32_t)nblob_ * blob_bytes2;
                         mbar_arrive_expect_tx(bar(kBarBFull + b_), bytes_);
-                        bulk_load(sbase + kOffB + b_ * kBPieceBytes, wset2 + (size_t)pc * st.c2_bpp * st.c2_blob_elems,
-                                  bytes_, bar(kBarBFull + b_));
+                        bulk_load(sbase + kOffB + b_ * kBPieceBytes, wset2 + (size_t)pc * ch.bpp2 * ch.blob2, bytes_,
+                                  bar(kBarBFull + b_));
                         wb.set_loaded(b_, -1, false);
                     }
                 }
-                if (!st.lookahead)
+                if (!ld.lookahead)
                     mbar_wait(bar(kBarAEmpty + (int)(a_cnt % kAStages)), ((a_cnt / kAStages) & 1u) ^ 1u, p.ctr,
                               pipe_limit, broken, 64);
-                next = (int)(atomicAdd(&p.ctr[MAFAT_CTR_TICKET], 1u) + gridDim.x);
-                if (next < p.n_items) it_next = p.items[next];
+                if (ld.lookahead != 2) mbar_arrive(bar(kBarTake));
             }
             // Drain: every copy issued has landed before the CTA may exit.
             for (uint32_t i = 0; i < kAStages && i < a_cnt; ++i) {
@@ -1449,7 +1318,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // chain item: the 3x3's accumulator goes to the epilogue, which writes its activated
                     // bf16 result back into TMEM; the chained 1x1 then runs from there
                     tc_commit_el(ms.el, ms.bar(kBarAccFull + buf));
-                    const ChainRec ch = recs[qs].chain;
+                    const MafatChainRec ch = recs[qs].chain;
                     mbar_arrive_el(ms.el, ms.bar(kBarQEmpty + qs));  // the slot is no longer read
                     const uint32_t mph = buf ? mid_ph1++ : mid_ph0++;
                     mbar_wait_mma(ms.bar(kBarMidFull + buf), mph & 1u, p.ctr, pipe_limit, broken);
@@ -1474,6 +1343,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         // scope).  The publisher's gpu-scope release reduction is cumulative over those
         // arrivals, so a consumer that acquires the counter sees every store; waiting for
         // the stores to reach L2 is this warp's job, not the epilogue warps'.
+        // Before that, the L2 prefetch: the input, the weights, the item records and scale / bias
+        // are read from DRAM once per run, mostly by loads that wait for them (the first layer's
+        // halos, the first use of every weight set and record on each SM); fetching them into
+        // L2 at once, spread over all CTAs, overlaps those DRAM latencies instead of paying them
+        // item by item.
+        if (lane < MAFAT_PF_REGIONS) prefetch_l2_share(p.pf_ptr[lane], p.pf_bytes[lane], p.pf_per[lane]);
+        __syncwarp();
         if (lane == 0) {
             uint32_t q_cnt = 0, e_cnt = 0;
             while (true) {
@@ -1511,7 +1387,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int qs = (int)(q_cnt % kQDepth);
             mbar_wait(bar(kBarQFull + qs), (q_cnt / kQDepth) & 1u, p.ctr, pipe_limit, broken, 256);
             const int ticket = q_items[qs];
-            GatherRec g{};
+            MafatGatherRec g{};
             int n_chunks = 0, rows_box = 0, rows = 0, cols = 0, hr = 0;
             if (ticket >= 0) {
                 g = recs[qs].gather;
@@ -1568,7 +1444,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int qs = (int)(q_cnt % kQDepth);
             mbar_wait(bar(kBarQFull + qs), (q_cnt / kQDepth) & 1u, p.ctr, pipe_limit, broken, 256);
             const int ticket = q_items[qs];
-            EpiRec rc;
+            MafatEpiRec rc;
             if (ticket >= 0) rc = recs[qs].epi;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarQEmpty + qs));
@@ -1618,6 +1494,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 bi += rc.n_mid;
             }
             const bool pool = (rc.flags & 1) != 0, nhwc = (rc.flags & 2) != 0;
+            const int out_kind = (rc.flags >> 4) & 7;
+            __nv_bfloat16* const out = (__nv_bfloat16*)(out_kind == MAFAT_BUF_USER_OUT ? p.user_out
+                                                        : out_kind == MAFAT_BUF_CUT    ? p.cut
+                                                                                       : p.scratch) + rc.out_off;
             // Work split between the warpgroups in units of one block x 32 output columns
             // (16 when N is an odd multiple of 16), dealt round-robin.
             const int uw = (rc.n_blk & 31) == 0 ? 32 : 16;
@@ -1650,7 +1530,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int Yw = yb + wq * 4 + 2 * (c & 1), Xw = xb + (c & ~1);
                     const uint32_t pix = (uint32_t)(((Yw >> 1) - rc.out_y0) * rc.out_w + ((Xw >> 1) - rc.out_x0));
                     EpiPoolDst pd;
-                    pd.out = rc.out;
+                    pd.out = out;
                     pd.nhwc = nhwc;
                     pd.pix = nhwc ? pix * (uint32_t)rc.cout : pix * 8u;
                     pd.plane = (uint32_t)(rc.out_h * rc.out_w * 8);
@@ -1678,7 +1558,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 const uint32_t pix = (uint32_t)((oy - rc.out_y0) * rc.out_w + (ox - rc.out_x0));
                 EpiDst dst;
-                dst.out = rc.out;
+                dst.out = out;
                 dst.nhwc = nhwc;
                 dst.pix = nhwc ? pix * (uint32_t)rc.cout : pix * 8u;
                 dst.plane = (uint32_t)(rc.out_h * rc.out_w * 8);

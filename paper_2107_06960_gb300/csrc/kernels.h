@@ -12,11 +12,10 @@ struct MafatKParams {
     const MafatStageDev* stages;
     const MafatTaskDev* tasks;
     const MafatItemDev* items;
+    const MafatItemRec* recs;     // bf16 path: item records in hand-out order (instead of the three tables)
     int32_t n_items;
     int32_t pad0;
     const CUtensorMap* tmaps;     // scratch-input and cut tensor maps (bf16 path)
-    int32_t cut_tmap;             // index of the cut tensor map (-1: none)
-    int32_t pad1;
     const uint16_t* w_bf16;       // packed tensor-core weights
     const float* w_f32;           // fp32 weights [cout][cin][k][k] per stage
     const float* scale;

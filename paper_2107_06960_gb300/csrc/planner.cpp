@@ -955,7 +955,7 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
         for (const MafatTaskDev& tk : t.tasks)
             if (tk.frame == 0) stage_items[tk.stage] += tk.n_items;
         for (size_t s = 0; s < t.stages.size(); ++s)
-            t.stages[s].lookahead = (cfg.lookahead_items >= 0 && stage_items[s] >= thr) ? 1 : 0;
+            t.stages[s].lookahead = (cfg.lookahead_items >= 0 && stage_items[s] >= thr) ? (reorder ? 2 : 1) : 0;
     }
     if (order.empty())
         for (int i = 0; i < (int)t.tasks.size(); ++i) order.push_back(i);
@@ -1252,6 +1252,106 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
         }
     }
     return "";
+}
+
+void build_records(const PlanTables& t, std::vector<MafatItemRec>& out) {
+    const int cut_map = t.cfg.n_groups >= 2 ? (int)t.tmaps.size() : -1;  // the cut tensor's map follows the others
+    out.assign(t.items.size(), MafatItemRec{});
+    for (size_t i = 0; i < t.items.size(); ++i) {
+        const MafatItemDev& it = t.items[i];
+        const MafatTaskDev& tk = t.tasks[it.task];
+        const MafatStageDev& st = t.stages[tk.stage];
+        MafatItemRec& r = out[i];
+        // a flat stage's item starts at pixel 128 by of its region read row by row: its A box starts
+        // at that pixel's row, the pixel being flat_off pixels into the box
+        int y_lo = 0, flat_off = -1;
+        if (st.flat) {
+            const int p0 = it.by * 128;
+            y_lo = p0 / st.cols_box;
+            flat_off = p0 - y_lo * st.cols_box;
+        }
+        MafatEpiRec& e = r.epi;
+        e.out_off = tk.out_off;
+        e.x0 = tk.cx0 + it.bx * MAFAT_BLK_COLS;
+        e.xlim = tk.cx0 + tk.cw;
+        e.y0 = (st.flat || st.blk_halo) ? tk.cy0 : tk.cy0 + it.by * MAFAT_BLK_ROWS;
+        e.ylim = tk.cy0 + tk.ch;
+        e.out_y0 = tk.out_y0;
+        e.out_x0 = tk.out_x0;
+        e.out_w = tk.out_w;
+        e.out_h = tk.out_h;
+        e.nbk = it.nbk;
+        e.nby = (int16_t)(st.blk_halo ? tk.nby : 0);
+        // what the epilogue stores: the item's own output, or a chain item's 1x1 output
+        e.n_blk = st.chain ? st.c2_n_blk : st.n_blk;
+        e.cout = st.chain ? st.c2_cout : st.cout;
+        e.ch_base = st.chain ? 0 : it.nb * st.n_blk;
+        e.flags = ((st.chain ? st.c2_pool : st.pool) ? 1 : 0) | (tk.out_nhwc ? 2 : 0) | ((it.flags & 1) ? 4 : 0) |
+                  (tk.out_kind << 4);
+        e.done_ctr = tk.done_ctr;
+        e.extra_ctr = it.extra_ctr;
+        e.chain = (int16_t)st.chain;
+        e.n_mid = (int16_t)st.n_blk;
+        e.a_col = (int16_t)st.chain_a_col;
+        e.out_col = (int16_t)st.chain_out_col;
+        e.pitch = (int16_t)(st.flat ? st.cols_box : 0);
+        e.flat_by = it.by;
+        uint32_t* w = r.mma.w;
+        w[0] = (uint32_t)(tk.stage * 256 + it.nb);
+        w[1] = (uint32_t)(st.sb_off + it.nb * st.n_blk);
+        w[2] = (uint32_t)(st.blob_elems * 2);
+        w[3] = (uint32_t)st.n_blk;
+        w[4] = (uint32_t)st.k | ((uint32_t)st.kst << 8) | ((uint32_t)it.nbk << 16) | ((uint32_t)st.paired << 24) |
+               ((uint32_t)st.b_swz << 25) | ((uint32_t)st.chain << 26) | ((uint32_t)st.pix_pair << 27) |
+               ((uint32_t)st.blk_halo << 28);
+        w[5] = (uint32_t)st.cols_box | ((uint32_t)st.rows_box << 16);
+        w[6] = (uint32_t)st.n_chunks | ((uint32_t)st.n_bsteps << 16);
+        w[7] = (uint32_t)st.bpp | ((uint32_t)st.n_pieces << 16);
+        w[8] = (uint32_t)(flat_off + 1) | ((uint32_t)(st.rows_box * st.cols_box) << 16);
+        if (st.chain) {
+            MafatChainRec& c = r.chain;
+            c.n2 = (int16_t)st.c2_n_blk;
+            c.nch2 = (int16_t)st.c2_n_chunks;
+            c.kst2 = (int16_t)st.c2_kst;
+            c.swz2 = (int16_t)st.c2_b_swz;
+            c.bpp2 = (int16_t)st.c2_bpp;
+            c.np2 = (int16_t)st.c2_n_pieces;
+            c.a_col = (int16_t)st.chain_a_col;
+            c.out_col = (int16_t)st.chain_out_col;
+            c.blob2 = st.c2_blob_elems;
+            c.sb2 = st.c2_sb_off;
+            c.w_off2 = st.c2_w_off;
+        }
+        MafatLoadRec& l = r.load;
+        const bool gather = tk.in_kind == MAFAT_BUF_USER_IN && st.in_mode == MAFAT_IN_GATHER;
+        const int px = tk.cx0 + it.bx * MAFAT_BLK_COLS - st.pad - tk.in_x0;  // first halo column
+        if (gather) {
+            const int e_start = px * st.cin;
+            r.gather.on = (int16_t)(st.pix_pair ? 2 : 1);
+            r.gather.c = (int16_t)st.cin;
+            r.gather.raw_e = (int16_t)st.raw_e;
+            r.gather.s0 = (int16_t)(e_start - (e_start & ~7));
+        }
+        l.dep0 = it.dep0;
+        l.dep0_target = it.dep0_target;
+        l.dep1 = it.dep1;
+        l.dep1_target = it.dep1_target;
+        l.task = it.task;
+        l.dep_first = tk.dep_first;
+        l.dep_count = tk.dep_count;
+        l.map = tk.in_kind == MAFAT_BUF_USER_IN ? -1 : tk.in_kind == MAFAT_BUF_CUT ? cut_map : tk.in_tmap;
+        l.w_off = st.w_off + (int64_t)it.nb * (st.set_bytes / 2);
+        l.x0 = gather ? px : px * 8;
+        l.y0 = tk.cy0 + (st.flat ? y_lo : gather ? 0 : it.by * MAFAT_BLK_ROWS) - st.pad - tk.in_y0;
+        l.c3 = tk.in_kind == MAFAT_BUF_SCRATCH ? 0 : tk.frame;
+        l.a_bytes = st.chunk8 * st.rows_box * st.cols_box * 16;
+        l.chunk8 = (int16_t)st.chunk8;
+        l.lookahead = (int16_t)st.lookahead;
+        l.g_nby = (int16_t)tk.nby;
+        l.g_by = it.by;
+        l.g_k = (int16_t)st.k;
+        l.g_cin = st.cin;
+    }
 }
 
 // Packed bf16 weight order, per stage: [n-block][chunk][blob], each blob one B operand of

@@ -165,6 +165,9 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
 // consists of items handed out earlier.  Returns "" or the first violation.
 std::string validate_plan(const Net& net, const PlanTables& t);
 
+// bf16 plans: the device record of every item (MafatItemRec), in hand-out order.
+void build_records(const PlanTables& t, std::vector<MafatItemRec>& out);
+
 // Pack fp32 weights [cout][cin][k][k] of every stage into the bf16 tensor-core
 // blob order (see pack_weights_bf16 in planner.cpp); out has weight_elems entries.
 void pack_weights_bf16(const Net& net, const PlanTables& t, std::vector<uint16_t>& out);

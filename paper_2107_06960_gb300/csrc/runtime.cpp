@@ -33,6 +33,7 @@ struct mafat_plan_s {
     MafatStageDev* d_stages = nullptr;
     MafatTaskDev* d_tasks = nullptr;
     MafatItemDev* d_items = nullptr;
+    MafatItemRec* d_recs = nullptr;  // bf16 plans: item records (in place of the stage, task and item tables)
     MafatDepDev* d_deps = nullptr;
     CUtensorMap* d_tmaps = nullptr;
     void* d_w = nullptr;
@@ -192,10 +193,10 @@ mafat_status launch(mafat_plan_s* p, const void* input, void* output, cudaStream
     kp.stages = p->d_stages;
     kp.tasks = p->d_tasks;
     kp.items = p->d_items;
+    kp.recs = p->d_recs;
     kp.deps = p->d_deps;
     kp.n_items = (int32_t)p->t.items.size();
     kp.tmaps = p->d_tmaps;
-    kp.cut_tmap = p->t.cfg.n_groups >= 2 ? (int)p->t.tmaps.size() : -1;
     kp.w_bf16 = (const uint16_t*)p->d_w;
     kp.w_f32 = (const float*)p->d_w;
     kp.scale = p->d_scale;
@@ -222,13 +223,12 @@ mafat_status launch(mafat_plan_s* p, const void* input, void* output, cudaStream
             in_dev = p->d_in_planar;
             in_dev_bytes = (int64_t)p->in_planar_bytes;
         }
-        const void* pf[] = {in_dev, p->d_w, p->d_items, p->d_tasks, p->d_stages, p->d_scale, p->d_bias};
+        const void* pf[] = {in_dev, p->d_w, p->d_recs, p->d_scale, p->d_bias};
         const int64_t pb[] = {in_dev_bytes, (int64_t)p->t.weight_elems * 2,
-                              (int64_t)(p->t.items.size() * sizeof(MafatItemDev)),
-                              (int64_t)(p->t.tasks.size() * sizeof(MafatTaskDev)),
-                              (int64_t)(p->t.stages.size() * sizeof(MafatStageDev)), (int64_t)p->t.sb_elems * 4,
+                              (int64_t)(p->t.items.size() * sizeof(MafatItemRec)), (int64_t)p->t.sb_elems * 4,
                               (int64_t)p->t.sb_elems * 4};
-        for (int i = 0; i < 7; ++i) {
+        static_assert(sizeof(pf) / sizeof(pf[0]) <= MAFAT_PF_REGIONS, "prefetch regions");
+        for (int i = 0; i < 5; ++i) {
             kp.pf_ptr[i] = pf[i];
             kp.pf_bytes[i] = pb[i];
             kp.pf_per[i] = ((pb[i] + p->grid - 1) / p->grid + 15) & ~(int64_t)15;
@@ -271,7 +271,6 @@ mafat_status mafat_internal_fp32_params(const mafat_plan_t* plan, MafatKParams* 
     k.deps = p->d_deps;
     k.n_items = (int32_t)p->t.items.size();
     k.tmaps = nullptr;
-    k.cut_tmap = -1;
     k.w_f32 = (const float*)p->d_w;
     k.scale = p->d_scale;
     k.bias = p->d_bias;
@@ -443,9 +442,21 @@ mafat_status mafat_plan_ex(const mafat_net_t* net, int32_t n_groups, const int32
         delete p;
         return cuda_fail(ee, what);
     };
-    if ((e = dalloc(p, &p->d_stages, t.stages.size() * sizeof(MafatStageDev))) != cudaSuccess) return bail(e, "cudaMalloc");
-    if ((e = dalloc(p, &p->d_tasks, t.tasks.size() * sizeof(MafatTaskDev))) != cudaSuccess) return bail(e, "cudaMalloc");
-    if ((e = dalloc(p, &p->d_items, t.items.size() * sizeof(MafatItemDev))) != cudaSuccess) return bail(e, "cudaMalloc");
+    if (dt == MAFAT_BF16) {
+        std::vector<MafatItemRec> recs;
+        mafat::build_records(t, recs);
+        if ((e = dalloc(p, &p->d_recs, recs.size() * sizeof(MafatItemRec))) != cudaSuccess) return bail(e, "cudaMalloc");
+        if ((e = cudaMemcpy(p->d_recs, recs.data(), recs.size() * sizeof(MafatItemRec), cudaMemcpyHostToDevice)) !=
+            cudaSuccess)
+            return bail(e, "cudaMemcpy");
+    } else {
+        if ((e = dalloc(p, &p->d_stages, t.stages.size() * sizeof(MafatStageDev))) != cudaSuccess) return bail(e, "cudaMalloc");
+        if ((e = dalloc(p, &p->d_tasks, t.tasks.size() * sizeof(MafatTaskDev))) != cudaSuccess) return bail(e, "cudaMalloc");
+        if ((e = dalloc(p, &p->d_items, t.items.size() * sizeof(MafatItemDev))) != cudaSuccess) return bail(e, "cudaMalloc");
+        if ((e = cudaMemcpy(p->d_stages, t.stages.data(), t.stages.size() * sizeof(MafatStageDev), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
+        if ((e = cudaMemcpy(p->d_tasks, t.tasks.data(), t.tasks.size() * sizeof(MafatTaskDev), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
+        if ((e = cudaMemcpy(p->d_items, t.items.data(), t.items.size() * sizeof(MafatItemDev), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
+                }
     if (!t.deps.empty()) {
         if ((e = dalloc(p, &p->d_deps, t.deps.size() * sizeof(MafatDepDev))) != cudaSuccess) return bail(e, "cudaMalloc");
         if ((e = cudaMemcpy(p->d_deps, t.deps.data(), t.deps.size() * sizeof(MafatDepDev), cudaMemcpyHostToDevice)) !=
@@ -476,9 +487,6 @@ mafat_status mafat_plan_ex(const mafat_net_t* net, int32_t n_groups, const int32
     }
     if ((e = cudaMemcpy(p->d_scale, sc.data(), sc.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
     if ((e = cudaMemcpy(p->d_bias, bi.data(), bi.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
-    if ((e = cudaMemcpy(p->d_stages, t.stages.data(), t.stages.size() * sizeof(MafatStageDev), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
-    if ((e = cudaMemcpy(p->d_tasks, t.tasks.data(), t.tasks.size() * sizeof(MafatTaskDev), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
-    if ((e = cudaMemcpy(p->d_items, t.items.data(), t.items.size() * sizeof(MafatItemDev), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
     if ((e = cudaMemset(p->d_scratch, 0, (size_t)p->scratch_bytes)) != cudaSuccess) return bail(e, "cudaMemset");
     if ((e = cudaMemset(p->d_ctr, 0, p->ctr_bytes)) != cudaSuccess) return bail(e, "cudaMemset");
     if (o.trace &&
