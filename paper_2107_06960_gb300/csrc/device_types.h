@@ -213,8 +213,9 @@ struct MafatEpiRec {
     int16_t n_mid;           // chain item: columns of the 3x3's accumulator
     int16_t a_col, out_col;  // chain item: TMEM columns of the 1x1's A operand and of its accumulator
     int16_t pitch;           // flat stage: row pitch of the region (pixels); 0: 16x8 blocks
-    int16_t flat_by;         // flat stage: the item's first block in the region; per-block-halo item:
-                             // its first block's index in the task's column-major block order
+    int16_t flat_by;         // flat stage: the item's first block in the region
+    int16_t by0, bx0;        // per-block-halo item: block row and column of its first block in the task
+    int32_t reserved[3];
 };
 
 // What the MMA issuer needs, packed in 32-bit words that it reads with three 16-byte
@@ -269,12 +270,11 @@ struct MafatLoadRec {
 };
 
 struct alignas(16) MafatItemRec {
-    MafatEpiRec epi;         // 80 bytes
+    MafatEpiRec epi;         // 96 bytes
     MafatMmaRec mma;         // 48
     MafatChainRec chain;     // 32
     MafatGatherRec gather;   // 8
     MafatLoadRec load;       // 72
-    int32_t reserved[4];
 };
 #define MAFAT_REC_BYTES 256
 static_assert(sizeof(MafatItemRec) == MAFAT_REC_BYTES, "item record");

@@ -42,11 +42,10 @@
 // accumulator's full barrier); TMEM: 2 accumulators of 256 columns (the epilogue
 // of one item overlaps the MMAs of the next).
 //
-// Epilogue: y = leaky_0.1(scale[n] * acc + bias[n]); for a fused 2x2/s2
-// max-pool the quad of pixels {(r, c), (r, c+1), (r+1, c), (r+1, c+1)} are lanes
-// {l, l^1, l^8, l^8^1} of one warp and are reduced with two shuffles; rounded
-// to bf16 (nearest-even) and stored to the tile's region buffer (octet-planar),
-// the cut tensor, or the NHWC output.
+// Epilogue: y = leaky_0.1(scale[n] * acc + bias[n]), rounded to bf16 (nearest-even) and stored to
+// the tile's region buffer (octet-planar), the cut tensor, or the NHWC output.  For a fused 2x2/s2
+// max-pool the two rows of a window are read into one lane and reduced before the scale is
+// applied, its two columns are neighbouring lanes and reduced with one shuffle.
 #include <cuda_bf16.h>
 
 #include "sched.cuh"
@@ -427,6 +426,21 @@ __device__ __forceinline__ void bn_leaky2(float s0, float s1, uint32_t a0, uint3
     v1 = fmaxf(z1, t1);
 }
 
+// The same in two steps: z = s * acc + b, then leaky ReLU and bf16 rounding.
+__device__ __forceinline__ void bn2(float s0, float s1, uint32_t a0, uint32_t a1, float b0, float b1, float& z0, float& z1) {
+    asm("{\n\t.reg .b64 s, a, b, z;\n\t"
+        "mov.b64 s, {%2, %3};\n\t"
+        "mov.b64 a, {%4, %5};\n\t"
+        "mov.b64 b, {%6, %7};\n\t"
+        "fma.rn.f32x2 z, s, a, b;\n\t"
+        "mov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(z0), "=f"(z1)
+        : "f"(s0), "f"(s1), "r"(a0), "r"(a1), "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ uint32_t leaky_bf16x2(float z0, float z1) {
+    return pack_bf16x2(fmaxf(z0, 0.1f * z0), fmaxf(z1, 0.1f * z1));
+}
+
 __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
     __nv_bfloat162 x = *reinterpret_cast<__nv_bfloat162*>(&a), y = *reinterpret_cast<__nv_bfloat162*>(&b);
     __nv_bfloat162 m = __hmax2(x, y);
@@ -446,100 +460,47 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Where one thread's epilogue results go: its pixel's element offset in the
-// output buffer (octet-planar: offset inside an 8-channel plane; NHWC: offset
-// of channel 0), the plane stride, and whether this lane stores at all.
-struct EpiDst {
-    __nv_bfloat16* out;
-    uint32_t pix, plane;  // element offsets within the output buffer (a frame's region: < 2^31)
-    int nhwc, cout, pool;
-    bool store;
-};
-
-// Epilogue of NC accumulator columns (output channels ch0 .. ch0+NC-1, NC = 16 or 32)
-// of one pixel per thread: folded BN, leaky ReLU 0.1 (as max(z, 0.1 z), the same value),
-// bf16 (nearest-even), 16-byte stores per octet of channels.
-//
-// A fused 2x2 max-pool reduces the window {(r, c), (r, c+1), (r+1, c), (r+1, c+1)},
-// lanes {l, l^1, l^8, l^9}, on packed bf16 pairs (rounding is monotonic, so the max of
-// rounded values is the rounded max) in two exchange rounds that each halve the octets a
-// lane holds: with the partner lane^1, a lane keeps octets 2m + (l & 1) and sends the
-// others; with lane^8, it keeps every other remaining octet.  Every shuffle carries data
-// both lanes need, and each lane of the window ends with its own octet(s) of the pooled
-// pixel to store (two octets: both lanes l and l^8 end with the same one; one stores).
-template <int NC>
-__device__ __forceinline__ void epi_chunk(uint32_t taddr, const float* sc, const float* bi, int ch0,
-                                          const EpiDst& d, int lane) {
-    static_assert(NC == 16 || NC == 32, "unit width");
-    constexpr int NO = NC / 8;  // octets
-    uint32_t raw[NC];
-    if constexpr (NC == 32)
-        tmem_ld32(taddr, raw);
-    else
-        tmem_ld16(taddr, raw);
-    uint32_t pk[NC / 2];
-#pragma unroll
-    for (int i = 0; i < NC; i += 4) {
-        const float4 s4 = *reinterpret_cast<const float4*>(sc + i);  // shared memory, same address
-        const float4 b4 = *reinterpret_cast<const float4*>(bi + i);  // for the whole warp
-        float v[4];
-        bn_leaky2(s4.x, s4.y, raw[i], raw[i + 1], b4.x, b4.y, v[0], v[1]);
-        bn_leaky2(s4.z, s4.w, raw[i + 2], raw[i + 3], b4.z, b4.w, v[2], v[3]);
-        pk[i / 2] = pack_bf16x2(v[0], v[1]);
-        pk[i / 2 + 1] = pack_bf16x2(v[2], v[3]);
-    }
-    if (!d.pool) {
-        if (!d.store) return;
-#pragma unroll
-        for (int o = 0; o < NO; ++o) {
-            const int ch = ch0 + 8 * o;
-            if (ch >= d.cout) break;  // channels past cout belong to the zero-padded MMA N
-            const uint4 w = make_uint4(pk[4 * o], pk[4 * o + 1], pk[4 * o + 2], pk[4 * o + 3]);
-            __nv_bfloat16* p = d.out + (d.nhwc ? d.pix + (uint32_t)ch : (uint32_t)(ch >> 3) * d.plane + d.pix);
-            *reinterpret_cast<uint4*>(p) = w;
-        }
-        return;
-    }
-    const bool h0 = (lane & 1) != 0, h3 = (lane & 8) != 0;
-    // first exchange, partner lane ^ 1: keep octet 2m + h0 of each pair (2m, 2m + 1)
-    uint32_t r1[NC / 4];
-#pragma unroll
-    for (int m = 0; m < NO / 2; ++m)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t lo = pk[8 * m + j], hi = pk[8 * m + 4 + j];
-            const uint32_t got = __shfl_xor_sync(0xffffffffu, h0 ? lo : hi, 1);
-            r1[4 * m + j] = max_bf16x2(h0 ? hi : lo, got);
-        }
-    if constexpr (NO == 4) {
-        // second exchange, partner lane ^ 8: keep octet 2 * h3 + h0
-        uint32_t r2[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t lo = r1[j], hi = r1[4 + j];
-            const uint32_t got = __shfl_xor_sync(0xffffffffu, h3 ? lo : hi, 8);
-            r2[j] = max_bf16x2(h3 ? hi : lo, got);
-        }
-        const int ch = ch0 + 8 * (2 * (int)h3 + (int)h0);
-        if (!d.store || ch >= d.cout) return;
-        __nv_bfloat16* p = d.out + (d.nhwc ? d.pix + (uint32_t)ch : (uint32_t)(ch >> 3) * d.plane + d.pix);
-        *reinterpret_cast<uint4*>(p) = make_uint4(r2[0], r2[1], r2[2], r2[3]);
-    } else {
-        // two octets: the second exchange is a plain max with lane ^ 8, and lanes with h3 set leave the store
-#pragma unroll
-        for (int j = 0; j < 4; ++j) r1[j] = max_bf16x2(r1[j], __shfl_xor_sync(0xffffffffu, r1[j], 8));
-        const int ch = ch0 + 8 * (int)h0;
-        if (!d.store || h3 || ch >= d.cout) return;
-        __nv_bfloat16* p = d.out + (d.nhwc ? d.pix + (uint32_t)ch : (uint32_t)(ch >> 3) * d.plane + d.pix);
-        *reinterpret_cast<uint4*>(p) = make_uint4(r1[0], r1[1], r1[2], r1[3]);
-    }
+// Epilogue loads of TMEM, valid after the next wait; the wait passes the registers through, so
+// that no use of them moves ahead of it.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr)
+                 : "memory");
 }
-
-// Sixteen TMEM lanes from `taddr` x 32 columns in the 16x256b shape (then wait): lane l of the
-// warp gets, for column group g = 0..3, v[4g + e] = column 8g + 2 (l % 4) + (e & 1) of TMEM lane
-// l / 4 (e < 2) or l / 4 + 8 (e >= 2) counted from taddr's lane (pinned on GB300 by a probe that
-// wrote lane << 8 | column into every cell).
-__device__ __forceinline__ void tmem_ld16x256_x4(uint32_t taddr, uint32_t (&v)[16]) {
+// Two groups of 16 TMEM lanes (taddr's and the 16 after them) x 8 columns in the 16x256b shape:
+// lane l of the warp gets v[4h + e] = column 2 (l % 4) + (e & 1) of TMEM lane 16 h + l / 4 (e < 2) or
+// 16 h + l / 4 + 8 (e >= 2) counted from taddr's lane (pinned on GB300 by a probe that wrote
+// lane << 8 | column into every cell).
+__device__ __forceinline__ void tmem_ld2x16x256(uint32_t taddr, uint32_t (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                 : "r"(taddr)
+                 : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+                 : "r"(taddr + (16u << 16))
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
+                 :
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr)
+        : "memory");
+}
+// 32 columns of the lanes as tmem_ld2x16x256: v[16h + 4g + e] = column 8g + 2 (l % 4) + (e & 1).
+__device__ __forceinline__ void tmem_ld2x16x256_x4(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
         "%15}, [%16];"
@@ -547,57 +508,36 @@ __device__ __forceinline__ void tmem_ld16x256_x4(uint32_t taddr, uint32_t (&v)[1
           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
         : "r"(taddr)
         : "memory");
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%16];"
+        : "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr + (16u << 16))
+        : "memory");
 }
-
-// Epilogue of one block x 32 accumulator columns (channels ch0 .. ch0 + 31) with the fused 2x2
-// max-pool, read in the 16x256b shape so that both rows of a pool window sit in one lane: the
-// warp's quarter holds conv rows 4 wq .. 4 wq + 3 of the block (TMEM lane = 8 row + column), and
-// its two loads (lanes +0 and +16) give lane l the pixels (2h, l / 4) and (2h + 1, l / 4) of
-// load h, channels 8g + 2 (l % 4) + {0, 1}.  Folded BN, leaky ReLU and bf16 rounding as in
-// epi_chunk, the vertical max in the lane, then one exchange with lane l ^ 4 (the next column):
-// a lane of an even column keeps pooled row 0 of its quarter, one of an odd column row 1.  Each
-// lane then stores 4 bytes (two channels) of each of its pooled pixel's four octets.
-struct EpiPoolDst {
-    __nv_bfloat16* out;
-    uint32_t pix, plane;  // element offset of the pooled pixel (NHWC: of its channel 0); octet plane
-    int nhwc, cout;
-    bool store;
-};
-__device__ __forceinline__ void epi_pool32(uint32_t taddr, const float* sc, const float* bi, int ch0,
-                                           const EpiPoolDst& d, int lane) {
-    uint32_t raw0[16], raw1[16];
-    tmem_ld16x256_x4(taddr, raw0);
-    tmem_ld16x256_x4(taddr + (16u << 16), raw1);
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    const int q2 = 2 * (lane & 3);
-    uint32_t pv0[4], pv1[4];  // per column group: bf16x2 of channels 8g + q2, + 1 after the vertical max
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        const float2 s = *reinterpret_cast<const float2*>(sc + 8 * g + q2);  // shared memory
-        const float2 c = *reinterpret_cast<const float2*>(bi + 8 * g + q2);
-        float a0, a1, b0, b1;
-        bn_leaky2(s.x, s.y, raw0[4 * g], raw0[4 * g + 1], c.x, c.y, a0, a1);
-        bn_leaky2(s.x, s.y, raw0[4 * g + 2], raw0[4 * g + 3], c.x, c.y, b0, b1);
-        pv0[g] = max_bf16x2(pack_bf16x2(a0, a1), pack_bf16x2(b0, b1));
-        bn_leaky2(s.x, s.y, raw1[4 * g], raw1[4 * g + 1], c.x, c.y, a0, a1);
-        bn_leaky2(s.x, s.y, raw1[4 * g + 2], raw1[4 * g + 3], c.x, c.y, b0, b1);
-        pv1[g] = max_bf16x2(pack_bf16x2(a0, a1), pack_bf16x2(b0, b1));
-    }
-    const bool odd = ((lane >> 2) & 1) != 0;
-    uint32_t res[4];
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? pv0[g] : pv1[g], 4);
-        res[g] = max_bf16x2(odd ? pv1[g] : pv0[g], got);
-    }
-    if (!d.store) return;
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-        const int ch = ch0 + 8 * g;
-        if (ch >= d.cout) break;  // channels past cout belong to the zero-padded MMA N
-        __nv_bfloat16* p = d.out + (d.nhwc ? d.pix + (uint32_t)(ch + q2) : (uint32_t)(ch >> 3) * d.plane + d.pix + q2);
-        *reinterpret_cast<uint32_t*>(p) = res[g];
-    }
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
+                   "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
+                   "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28])
+                 :
+                 : "memory");
+    asm volatile("" : "+r"(v[29]), "+r"(v[30]), "+r"(v[31]) : : "memory");
+}
+// Stores under a predicate, without a branch.
+__device__ __forceinline__ void st16_if(bool on, __nv_bfloat16* p, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t@p st.global.v4.b32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"((int)on),
+                 "l"(p), "r"(a), "r"(b), "r"(c), "r"(d)
+                 : "memory");
+}
+__device__ __forceinline__ void st4_if(bool on, __nv_bfloat16* p, uint32_t a) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %0, 0;\n\t@p st.global.b32 [%1], %2;\n\t}" ::"r"((int)on), "l"(p), "r"(a)
+                 : "memory");
+}
+__device__ __forceinline__ float max_f32(uint32_t a, uint32_t b) {
+    return fmaxf(__uint_as_float(a), __uint_as_float(b));
 }
 
 // Weight-buffer bookkeeping.  The producer and the MMA issuer each keep a copy and
@@ -1500,75 +1440,172 @@ __global__ void __launch_bounds__(kThreads, 1)
                                                                                        : p.scratch) + rc.out_off;
             // Work split between the warpgroups in units of one block x 32 output columns
             // (16 when N is an odd multiple of 16), dealt round-robin.
-            const int uw = (rc.n_blk & 31) == 0 ? 32 : 16;
+            const bool wide = (rc.n_blk & 31) == 0;
             // units per block (at least 1: only a record read after a pipeline wait ran out
-            // can hold a smaller N, and the unit walk below must end)
-            const int upb = max(1, uw == 32 ? rc.n_blk >> 5 : rc.n_blk >> 4);
-            // unit u = b * upb + qi, from u = h in steps of kEpiGroups (no division per unit)
-            for (int b = 0, qi = h;; qi += kEpiGroups) {
-                while (qi >= upb) {
-                    qi -= upb;
-                    ++b;
+            // can hold a smaller N, and the walk below must end)
+            const int upb = max(1, wide ? rc.n_blk >> 5 : rc.n_blk >> 4);
+            const uint32_t plane = (uint32_t)(rc.out_h * rc.out_w * 8);
+            const uint32_t acc0 = acc_lanes + col0;
+            // octet o of channels starts at this element offset from the pixel's
+            const uint32_t oct = nhwc ? 8u : plane, pix_el = nhwc ? (uint32_t)rc.cout : 8u;
+            int b = 0, qi = h;                                        // block of the item, unit of the block
+            int Y = rc.y0 + (rc.nby > 0 ? rc.by0 * MAFAT_BLK_ROWS : 0);  // conv position of the block's first pixel
+            int X = rc.x0 + (rc.nby > 0 ? rc.bx0 * MAFAT_BLK_COLS : 0);
+            const int y_wrap = rc.nby > 0 ? rc.y0 + rc.nby * MAFAT_BLK_ROWS : 0x7fffffff;
+            // The unit after (b, qi), without branches: a unit's code is one straight run, because each
+            // scheduler has two epilogue warps to issue from, and branches (per octet, per store, per
+            // step) left them fetching instructions.  Measured on GB300, first layer of 608x608: 0.65
+            // us a unit with them, 0.40 without, whatever its loads, shuffles and arithmetic cost
+            // (each taken out in turn changed nothing; a rolled loop over octets took 0.85).  The two
+            // steps cover the two warpgroups.
+            auto advance = [&](int step) {
+                qi += step;
+#pragma unroll
+                for (int i = 0; i < kEpiGroups; ++i) {
+                    const bool next = qi >= upb;  // on to the next block
+                    qi -= next ? upb : 0;
+                    b += next ? 1 : 0;
+                    Y += next ? MAFAT_BLK_ROWS : 0;
+                    const bool wrap = Y >= y_wrap;  // per-block halos: the blocks run down the task's block columns
+                    Y = wrap ? rc.y0 : Y;
+                    X += wrap ? MAFAT_BLK_COLS : 0;
                 }
-                if (b >= rc.nbk) break;
-                const int q = qi * uw;
-                const uint32_t taddr = acc_lanes + col0 + (uint32_t)(b * rc.n_blk + q);
-                // conv position of the block's top-left pixel
-                int yb = rc.y0 + b * MAFAT_BLK_ROWS, xb = rc.x0;
-                if (rc.nby > 0) {
-                    // per-block halos: the item's block b is block flat_by + b of its task in
-                    // column-major order
-                    const int lin = rc.flat_by + b;
-                    const int bxx = lin / rc.nby;
-                    yb = rc.y0 + (lin - bxx * rc.nby) * MAFAT_BLK_ROWS;
-                    xb = rc.x0 + bxx * MAFAT_BLK_COLS;
-                }
-                if (pool && uw == 32) {
-                    // the window of this lane's pooled pixel (epi_pool32): rows 4 wq + 2 (c & 1) + {0, 1},
-                    // columns (c & ~1) + {0, 1} of the block, c = lane / 4
-                    const int c = lane >> 2;
-                    const int Yw = yb + wq * 4 + 2 * (c & 1), Xw = xb + (c & ~1);
+            };
+            advance(0);
+            if (wide && pool) {
+                // Pooled units: 16x256b loads put both rows of a pool window in one lane: the warp's
+                // quarter holds conv rows 4 wq .. 4 wq + 3 of the block (TMEM lane = 8 row + column), and
+                // lane l gets pixels (2h, l / 4) and (2h + 1, l / 4) of load h, channels 8g + 2 (l % 4) +
+                // {0, 1}.  The vertical maximum is taken on the accumulators: a pooled stage's scales
+                // are not negative (their sign is in the packed weights), so scale, bias, leaky ReLU
+                // and rounding are monotonic and the maximum of the results is the result of the
+                // maximum, for half the arithmetic.  One exchange with lane l ^ 4 (the next column): a
+                // lane of an even column keeps pooled row 0 of its quarter, one of an odd column row 1,
+                // and stores 4 bytes (two channels) of each of its pooled pixel's four octets.
+                const int q2 = 2 * (lane & 3), c = lane >> 2;
+                const bool odd = (c & 1) != 0;
+                uint32_t v[32];
+                if (b < rc.nbk) tmem_ld2x16x256_x4(acc0 + (uint32_t)(b * rc.n_blk + qi * 32), v);
+#pragma unroll 1
+                while (b < rc.nbk) {
+                    const int q = qi * 32, ch = rc.ch_base + q;
+                    const int Yw = Y + wq * 4 + 2 * (c & 1), Xw = X + (c & ~1);
+                    const bool store = Yw < rc.ylim && Xw < rc.xlim;
                     const uint32_t pix = (uint32_t)(((Yw >> 1) - rc.out_y0) * rc.out_w + ((Xw >> 1) - rc.out_x0));
-                    EpiPoolDst pd;
-                    pd.out = out;
-                    pd.nhwc = nhwc;
-                    pd.pix = nhwc ? pix * (uint32_t)rc.cout : pix * 8u;
-                    pd.plane = (uint32_t)(rc.out_h * rc.out_w * 8);
-                    pd.cout = rc.cout;
-                    pd.store = (Yw < rc.ylim) && (Xw < rc.xlim);
-                    epi_pool32(taddr, sc + q, bi + q, rc.ch_base + q, pd, lane);
-                    continue;
+                    __nv_bfloat16* const dst = out + (size_t)(pix * pix_el + (uint32_t)(ch >> 3) * oct + (uint32_t)q2);
+                    float2 s[4], bs[4];
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        s[g] = *reinterpret_cast<const float2*>(sc + q + 8 * g + q2);
+                        bs[g] = *reinterpret_cast<const float2*>(bi + q + 8 * g + q2);
+                    }
+                    tmem_ld_wait(v);
+                    float m[16];  // per column group: pooled row 0's two channels, row 1's
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            m[4 * g + i] = max_f32(v[16 * (i >> 1) + 4 * g + (i & 1)], v[16 * (i >> 1) + 4 * g + (i & 1) + 2]);
+                    advance(kEpiGroups);
+                    // after the last unit the load is repeated on the item's first block (never used)
+                    tmem_ld2x16x256_x4(acc0 + (b < rc.nbk ? (uint32_t)(b * rc.n_blk + qi * 32) : 0u), v);
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        float z0, z1, y0, y1;
+                        bn2(s[g].x, s[g].y, __float_as_uint(m[4 * g]), __float_as_uint(m[4 * g + 1]), bs[g].x, bs[g].y, z0, z1);
+                        bn2(s[g].x, s[g].y, __float_as_uint(m[4 * g + 2]), __float_as_uint(m[4 * g + 3]), bs[g].x, bs[g].y, y0, y1);
+                        const uint32_t p0 = leaky_bf16x2(z0, z1), p1 = leaky_bf16x2(y0, y1);
+                        const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? p0 : p1, 4);
+                        // channels past cout belong to the zero-padded MMA N
+                        st4_if(store && ch + 8 * g < rc.cout, dst + (size_t)g * oct, max_bf16x2(odd ? p1 : p0, got));
+                    }
                 }
-                int Y = yb + r, Xb = xb + cc;
-                if (rc.pitch > 0) {
-                    // flat stage (never pooled): pixel 128 (flat_by + b) + 32 wq + lane of the
-                    // region read row after row, rc.pitch pixels a row
-                    const int pf = (rc.flat_by + b) * 128 + wq * 32 + lane;
-                    const int yy = pf / rc.pitch;
-                    Y = rc.y0 + yy;
-                    Xb = rc.x0 + (pf - yy * rc.pitch);
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            } else if (wide) {
+                // One pixel per thread, 32 channels per unit: a 16-byte store per octet.
+                uint32_t v[32];
+#pragma unroll 1
+                while (b < rc.nbk) {
+                    const int q = qi * 32, ch = rc.ch_base + q;
+                    tmem_ld32_async(acc0 + (uint32_t)(b * rc.n_blk + q), v);
+                    int Yp = Y + r, Xp = X + cc;
+                    if (rc.pitch > 0) {
+                        // flat stage: pixel 128 (flat_by + b) + 32 wq + lane of the region read row after
+                        // row, rc.pitch pixels a row
+                        const int pf = (rc.flat_by + b) * 128 + wq * 32 + lane;
+                        const int yy = pf / rc.pitch;
+                        Yp = rc.y0 + yy;
+                        Xp = rc.x0 + (pf - yy * rc.pitch);
+                    }
+                    const bool store = Yp < rc.ylim && Xp < rc.xlim;
+                    const uint32_t pix = (uint32_t)((Yp - rc.out_y0) * rc.out_w + (Xp - rc.out_x0));
+                    __nv_bfloat16* const dst = out + (size_t)(pix * pix_el + (uint32_t)(ch >> 3) * oct);
+                    tmem_ld_wait(v);
+                    float z[32];
+#pragma unroll
+                    for (int i = 0; i < 32; i += 4) {
+                        const float4 s4 = *reinterpret_cast<const float4*>(sc + q + i);  // shared memory, same address
+                        const float4 b4 = *reinterpret_cast<const float4*>(bi + q + i);  // for the whole warp
+                        bn2(s4.x, s4.y, v[i], v[i + 1], b4.x, b4.y, z[i], z[i + 1]);
+                        bn2(s4.z, s4.w, v[i + 2], v[i + 3], b4.z, b4.w, z[i + 2], z[i + 3]);
+                    }
+                    advance(kEpiGroups);
+#pragma unroll
+                    for (int o = 0; o < 4; ++o)
+                        st16_if(store && ch + 8 * o < rc.cout, dst + (size_t)o * oct, leaky_bf16x2(z[8 * o], z[8 * o + 1]),
+                                leaky_bf16x2(z[8 * o + 2], z[8 * o + 3]), leaky_bf16x2(z[8 * o + 4], z[8 * o + 5]),
+                                leaky_bf16x2(z[8 * o + 6], z[8 * o + 7]));
                 }
-                const bool valid = (Y < rc.ylim) && (Xb < rc.xlim);
-                // a pooled stage's conv region starts on even rows and columns and has even
-                // extents, so a window's four lanes agree on valid
-                int oy = Y, ox = Xb;
-                if (pool) {
-                    oy = Y >> 1;
-                    ox = Xb >> 1;
+            } else {
+                // N an odd multiple of 16: eight columns at a time, pooled or not
+                const int q2 = 2 * (lane & 3), c = lane >> 2;
+                const bool odd = (c & 1) != 0;
+                while (b < rc.nbk) {
+#pragma unroll 1
+                    for (int k = 0; k < 16; k += 8) {
+                        const int col = qi * 16 + k, ch = rc.ch_base + col;
+                        const uint32_t taddr = acc0 + (uint32_t)(b * rc.n_blk + col);
+                        uint32_t v[8];
+                        if (pool) {
+                            tmem_ld2x16x256(taddr, v);
+                            tmem_ld_wait(v);
+                            const float2 s2 = *reinterpret_cast<const float2*>(sc + col + q2);
+                            const float2 b2 = *reinterpret_cast<const float2*>(bi + col + q2);
+                            float z0, z1, y0, y1;
+                            bn2(s2.x, s2.y, __float_as_uint(max_f32(v[0], v[2])), __float_as_uint(max_f32(v[1], v[3])), b2.x, b2.y, z0, z1);
+                            bn2(s2.x, s2.y, __float_as_uint(max_f32(v[4], v[6])), __float_as_uint(max_f32(v[5], v[7])), b2.x, b2.y, y0, y1);
+                            const uint32_t p0 = leaky_bf16x2(z0, z1), p1 = leaky_bf16x2(y0, y1);
+                            const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? p0 : p1, 4);
+                            const int Yw = Y + wq * 4 + 2 * (c & 1), Xw = X + (c & ~1);
+                            const uint32_t pix = (uint32_t)(((Yw >> 1) - rc.out_y0) * rc.out_w + ((Xw >> 1) - rc.out_x0));
+                            st4_if(Yw < rc.ylim && Xw < rc.xlim && ch < rc.cout,
+                                   out + (size_t)(pix * pix_el + (uint32_t)(ch >> 3) * oct + (uint32_t)q2), max_bf16x2(odd ? p1 : p0, got));
+                        } else {
+                            tmem_ld8(taddr, v);
+                            tmem_ld_wait(v);
+                            int Yp = Y + r, Xp = X + cc;
+                            if (rc.pitch > 0) {
+                                const int pf = (rc.flat_by + b) * 128 + wq * 32 + lane;
+                                const int yy = pf / rc.pitch;
+                                Yp = rc.y0 + yy;
+                                Xp = rc.x0 + (pf - yy * rc.pitch);
+                            }
+                            const uint32_t pix = (uint32_t)((Yp - rc.out_y0) * rc.out_w + (Xp - rc.out_x0));
+                            uint32_t w[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const float2 s2 = *reinterpret_cast<const float2*>(sc + col + 2 * i);
+                                const float2 b2 = *reinterpret_cast<const float2*>(bi + col + 2 * i);
+                                float z0, z1;
+                                bn2(s2.x, s2.y, v[2 * i], v[2 * i + 1], b2.x, b2.y, z0, z1);
+                                w[i] = leaky_bf16x2(z0, z1);
+                            }
+                            st16_if(Yp < rc.ylim && Xp < rc.xlim && ch < rc.cout,
+                                    out + (size_t)(pix * pix_el + (uint32_t)(ch >> 3) * oct), w[0], w[1], w[2], w[3]);
+                        }
+                    }
+                    advance(kEpiGroups);
                 }
-                const uint32_t pix = (uint32_t)((oy - rc.out_y0) * rc.out_w + (ox - rc.out_x0));
-                EpiDst dst;
-                dst.out = out;
-                dst.nhwc = nhwc;
-                dst.pix = nhwc ? pix * (uint32_t)rc.cout : pix * 8u;
-                dst.plane = (uint32_t)(rc.out_h * rc.out_w * 8);
-                dst.cout = rc.cout;
-                dst.store = valid;
-                dst.pool = pool;
-                if (uw == 32)
-                    epi_chunk<32>(taddr, sc + q, bi + q, rc.ch_base + q, dst, lane);
-                else
-                    epi_chunk<16>(taddr, sc + q, bi + q, rc.ch_base + q, dst, lane);
             }
             tc_fence_before();
             mbar_arrive(bar(kBarAccEmpty + buf));  // also frees the scale / bias slot

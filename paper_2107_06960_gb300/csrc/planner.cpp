@@ -2,6 +2,7 @@
 #include "planner.h"
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <string>
 
@@ -1296,6 +1297,10 @@ void build_records(const PlanTables& t, std::vector<MafatItemRec>& out) {
         e.out_col = (int16_t)st.chain_out_col;
         e.pitch = (int16_t)(st.flat ? st.cols_box : 0);
         e.flat_by = it.by;
+        if (st.blk_halo) {
+            e.bx0 = (int16_t)(it.by / tk.nby);
+            e.by0 = (int16_t)(it.by - e.bx0 * tk.nby);
+        }
         uint32_t* w = r.mma.w;
         w[0] = (uint32_t)(tk.stage * 256 + it.nb);
         w[1] = (uint32_t)(st.sb_off + it.nb * st.n_blk);
@@ -1369,6 +1374,8 @@ void build_records(const PlanTables& t, std::vector<MafatItemRec>& out) {
 //  - pixel-pair stages (3x3, at most 4 input channels): blob p is kernel row ky = p; K half h
 //    holds taps kx = 2h (elements 0-3, its channels) and 2h + 1 (elements 4-7; kx = 3 is a
 //    zero tap), matching a halo slot that holds two neighbouring pixels of 4 channels.
+// In a stage with a fused pool the scale's sign is moved into the channel's weights (exact), so
+// that the epilogue may take the maximum of accumulators before it applies a scale >= 0.
 void pack_weights_bf16(const Net& net, const PlanTables& t, std::vector<uint16_t>& out) {
     out.assign((size_t)t.weight_elems, 0);
     for (const MafatStageDev& s : t.stages) {
@@ -1407,13 +1414,19 @@ void pack_weights_bf16(const Net& net, const PlanTables& t, std::vector<uint16_t
                                 from[e] = tap >= 0 && ci < cin ? ci * taps + tap : -1;
                             }
                             const float* src = w.data() + (size_t)nb * s.n_blk * cin * taps;
+                            const float* scale = net.scale[s.layer].data() + nb * s.n_blk;
                             for (int nn = 0; nn < n; ++nn, src += (size_t)cin * taps) {
+                                // a pooled stage: the sign of the scale goes into the weights (none
+                                // for a zero scale), pack_scale_bias keeps its magnitude
+                                const uint16_t flip = s.pool && scale[nn] < 0.f ? 0x8000u : 0u;
+                                const bool zero = s.pool && scale[nn] == 0.f;
                                 // swizzled: 16-byte unit 2j + h of the channel's 128-byte row
                                 uint16_t* dst = out.data() + blob +
                                                 (s.b_swz ? (size_t)(nn / 8) * 512 + (size_t)(nn % 8) * 64 +
                                                                (size_t)(((2 * j + h) ^ (nn % 8)) * 8)
                                                          : ((size_t)j * 2 + h) * s.n_blk * 8 + (size_t)nn * 8);
-                                for (int e = 0; e < 8; ++e) dst[e] = from[e] >= 0 ? f32_to_bf16_rne(src[from[e]]) : 0;
+                                for (int e = 0; e < 8; ++e)
+                                    dst[e] = from[e] >= 0 && !zero ? (uint16_t)(f32_to_bf16_rne(src[from[e]]) ^ flip) : 0;
                             }
                         }
                 }
@@ -1445,6 +1458,8 @@ void pack_scale_bias(const Net& net, const PlanTables& t, std::vector<float>& sc
     bias.assign((size_t)t.sb_elems, 0.f);
     for (const MafatStageDev& s : t.stages) {
         std::copy(net.scale[s.layer].begin(), net.scale[s.layer].end(), scale.begin() + s.sb_off);
+        if (t.cfg.dtype == 0 && s.pool)  // the sign is in the packed weights (pack_weights_bf16)
+            for (int o = 0; o < s.cout; ++o) scale[s.sb_off + o] = std::fabs(scale[s.sb_off + o]);
         std::copy(net.bias[s.layer].begin(), net.bias[s.layer].end(), bias.begin() + s.sb_off);
     }
 }
