@@ -227,8 +227,8 @@ __device__ __forceinline__ void mbar_arrive_el(uint32_t el, uint32_t bar) {
         : "memory");
 }
 
-// The loader's forms of the above: all lanes run them in step and the one with el = 1 acts, so
-// that the loader's loop stays converged and free of branches on the lane (measured on GB300
+// The loader's and the publisher's forms of the above: all lanes run them in step and the one with el = 1 acts, so
+// that their loops stay converged and free of branches on the lane (measured on GB300
 // against a loop of lane 0 alone: 16 608x608 frames 815 -> 765 us, one 90.3 -> 86.5).
 __device__ __forceinline__ void mbar_arrive_expect_tx_el(uint32_t el, uint32_t bar, uint32_t bytes) {
     asm volatile(
@@ -253,6 +253,11 @@ __device__ __forceinline__ void tma_load_3d_el(uint32_t el, uint32_t dst, const 
         " [%0], [%1, {%2, %3, %4}], [%5];\n\t}" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar), "r"(el)
         : "memory");
+}
+__device__ __forceinline__ void red_release_add_el(uint32_t el, uint32_t* p) {
+    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t@e red.release.gpu.global.add.u32 [%0], 1;\n\t}" ::"l"(p),
+                 "r"(el)
+                 : "memory");
 }
 __device__ __forceinline__ void bulk_load_el(uint32_t el, uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
     asm volatile(
@@ -1299,26 +1304,25 @@ __global__ void __launch_bounds__(kThreads, 1)
         // item by item.
         if (lane < MAFAT_PF_REGIONS) prefetch_l2_share(p.pf_ptr[lane], p.pf_bytes[lane], p.pf_per[lane]);
         __syncwarp();
-        if (lane == 0) {
+        {
+            const uint32_t el = elect_one();
             uint32_t q_cnt = 0, e_cnt = 0;
             while (true) {
                 const int qs = (int)(q_cnt % kQDepth);
                 mbar_wait(bar(kBarQFull + qs), (q_cnt / kQDepth) & 1u, p.ctr, pipe_limit, broken, 256);
                 const int ticket = q_items[qs];
-                int done_ctr = 0, extra_ctr = -1, flags = 0;
-                if (ticket >= 0) {
-                    done_ctr = recs[qs].epi.done_ctr;
-                    extra_ctr = recs[qs].epi.extra_ctr;
-                    flags = recs[qs].epi.flags;
-                }
-                mbar_arrive(bar(kBarQEmpty + qs));
+                const int done_ctr = recs[qs].epi.done_ctr, extra_ctr = recs[qs].epi.extra_ctr, flags = recs[qs].epi.flags;
+                __syncwarp();  // every lane has read its copy
+                mbar_arrive_el(el, bar(kBarQEmpty + qs));
                 ++q_cnt;
                 if (ticket < 0) break;
                 const int es = (int)(e_cnt & 1u);
                 mbar_wait(bar(kBarEpiDone + es), (e_cnt >> 1) & 1u, p.ctr, pipe_limit, broken);
-                if (!(flags & 4)) mafat_dev::publish_counters(p.ctr, done_ctr, extra_ctr);
-                if (trace) mafat_dev::trace_put(trace, ticket, 3, mafat_dev::globaltimer_ns());
-                mbar_arrive(bar(kBarPubDone + es));
+                const uint32_t pub = (flags & 4) ? 0u : el;
+                red_release_add_el(pub, p.ctr + done_ctr);
+                red_release_add_el(extra_ctr >= 0 ? pub : 0u, p.ctr + max(extra_ctr, 0));
+                if (trace && lane == 0) mafat_dev::trace_put(trace, ticket, 3, mafat_dev::globaltimer_ns());
+                mbar_arrive_el(el, bar(kBarPubDone + es));
                 ++e_cnt;
             }
         }
