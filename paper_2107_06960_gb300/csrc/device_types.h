@@ -206,8 +206,8 @@ struct MafatEpiRec {
     int16_t nby;             // per-block-halo item: block rows of its task (0: blocks stacked from y0)
     int32_t n_blk;           // output channels per item (accumulator columns per block)
     int32_t cout, ch_base;   // channels of the layer; first channel of the item
-    int32_t flags;           // bit 0: fused max-pool, bit 1: NHWC output, bit 2: never published (test
-                             // hook), bits 4-6: MAFAT_BUF_* of the output
+    int32_t flags;           // bit 0: fused max-pool, bit 1: NHWC output, bit 2: not published (nothing
+                             // waits for it, or the test hook), bits 4-6: MAFAT_BUF_* of the output
     int32_t done_ctr, extra_ctr;
     int16_t chain;           // 1: chain item (first pass turns the 3x3's result into the 1x1's A operand)
     int16_t n_mid;           // chain item: columns of the 3x3's accumulator

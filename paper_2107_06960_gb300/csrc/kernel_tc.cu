@@ -89,6 +89,7 @@ constexpr int kRecStride = MAFAT_REC_BYTES;
 constexpr int kOffQItems = kOffRec + kQDepth * kRecStride;
 constexpr int kOffTmem = kOffQItems + 4 * kQDepth;
 constexpr int kOffBroken = kOffTmem + 4;
+constexpr int kOffExited = kOffBroken + 4;         // 1: this CTA has counted itself out (finish_warp)
 constexpr int kOffA = 2048;
 constexpr int kOffB = kOffA + kAStages * kAStageBytes;
 constexpr int kSbSlotBytes = 2 * MAFAT_MAX_NBLK * 4;  // scale then bias of one item's channels
@@ -96,7 +97,7 @@ constexpr int kOffSb = kOffB + 2 * kBPieceBytes;
 constexpr int kSmemUsed = kOffSb + 2 * kSbSlotBytes;
 constexpr int kSmemBytes = kSmemUsed + 1024;  // slack for aligning the base
 static_assert(kNumBars * 8 <= kOffRec, "barrier area");
-static_assert(kOffBroken + 4 <= kOffA, "queue area");
+static_assert(kOffExited + 4 <= kOffA, "queue area");
 static_assert(kSmemBytes <= 232448, "shared memory");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -904,6 +905,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile int* q_items = reinterpret_cast<volatile int*>(smem + kOffQItems);
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kOffTmem);
     volatile int* broken = reinterpret_cast<volatile int*>(smem + kOffBroken);
+    volatile int* exited = reinterpret_cast<volatile int*>(smem + kOffExited);
     MafatItemRec* recs = reinterpret_cast<MafatItemRec*>(smem + kOffRec);
     auto bar = [&](int i) { return sbase + (uint32_t)(i * 8); };
 
@@ -942,6 +944,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(bar(kBarPubDone + i), 1);
         }
         *broken = 0;
+        *exited = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kMmaWarp) {
@@ -1325,6 +1328,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 mbar_arrive_el(el, bar(kBarPubDone + es));
                 ++e_cnt;
             }
+            // Every item of the CTA has been published and no further ticket will be taken: count the
+            // CTA out here, beside the other warps' last steps.  (After a pipeline wait ran out the
+            // roles may be out of step: then at the end, once all of them are done.)
+            if (__any_sync(0xffffffffu, *broken != 0) == 0) {
+                mafat_dev::finish_warp(p.ctr, p.n_ctr, lane);
+                if (lane == 0) *exited = 1;
+            }
         }
         __syncwarp();
     } else if (warp == kGatherWarp) {
@@ -1641,7 +1651,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols)
                      : "memory");
     }
-    mafat_dev::finish_cta(p.ctr, p.n_ctr);
+    if (*exited == 0) mafat_dev::finish_cta(p.ctr, p.n_ctr);  // (the same for every thread)
 }
 
 // ---------------------------------------------------------------------------

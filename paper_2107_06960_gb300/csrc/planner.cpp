@@ -1258,6 +1258,13 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
 void build_records(const PlanTables& t, std::vector<MafatItemRec>& out) {
     const int cut_map = t.cfg.n_groups >= 2 ? (int)t.tmaps.size() : -1;  // the cut tensor's map follows the others
     out.assign(t.items.size(), MafatItemRec{});
+    // tasks whose completion some item waits for; the others' items need not be published (a
+    // publication waits ~0.65 us for the item's stores to reach L2, at the end of the launch)
+    std::vector<char> awaited(t.tasks.size(), 0);
+    for (const MafatItemDev& it : t.items)
+        for (int ctr : {it.dep0, it.dep1})
+            if (ctr >= MAFAT_CTR_BASE && ctr < t.frame_ctr_base) awaited[ctr - MAFAT_CTR_BASE] = 1;
+    for (const MafatDepDev& d : t.deps) awaited[d.ctr - MAFAT_CTR_BASE] = 1;
     for (size_t i = 0; i < t.items.size(); ++i) {
         const MafatItemDev& it = t.items[i];
         const MafatTaskDev& tk = t.tasks[it.task];
@@ -1288,7 +1295,7 @@ void build_records(const PlanTables& t, std::vector<MafatItemRec>& out) {
         e.cout = st.chain ? st.c2_cout : st.cout;
         e.ch_base = st.chain ? 0 : it.nb * st.n_blk;
         e.flags = ((st.chain ? st.c2_pool : st.pool) ? 1 : 0) | (tk.out_nhwc ? 2 : 0) | ((it.flags & 1) ? 4 : 0) |
-                  (tk.out_kind << 4);
+                  (!awaited[it.task] && it.extra_ctr < 0 ? 4 : 0) | (tk.out_kind << 4);
         e.done_ctr = tk.done_ctr;
         e.extra_ctr = it.extra_ctr;
         e.chain = (int16_t)st.chain;

@@ -126,6 +126,19 @@ __device__ __forceinline__ void trace_put(unsigned long long* tr, int ticket, in
     if (tr) tr[(size_t)ticket * MAFAT_TRACE_WORDS + field] = v;
 }
 
+// Called by one warp, all lanes, after its CTA's last use of the counters (its publications and
+// everything they follow): the last CTA of the launch to get here zeroes the counter block (all
+// but the status word) for the next run on the same stream.
+__device__ __forceinline__ void finish_warp(uint32_t* ctr, int n_ctr, int lane) {
+    uint32_t done = 0;
+    if (lane == 0)  // release: this CTA's publications come first; acquire: so do the others'
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(done) : "l"(ctr + MAFAT_CTR_EXIT) : "memory");
+    done = __shfl_sync(0xffffffffu, done, 0);
+    if (done != gridDim.x - 1) return;
+    for (int i = lane; i < n_ctr; i += 32)
+        if (i != MAFAT_CTR_STATUS) ctr[i] = 0u;
+}
+
 // Called by every thread of a CTA after its last use of the counters: the last
 // CTA of the launch to get here zeroes the counter block (all but the status
 // word) for the next run on the same stream.
