@@ -265,16 +265,27 @@ int f32_region_items(const MafatStageDev& s, int ch, int cw) {
 }
 
 // Shape of an fp32 stage's items.  A thread computes 8 pixels x f32_ct channels, the CTA's 128
-// threads f32_groups x 8 pixels x 8, 16, 32 or 64 channels.  A chunk of a 3x3 costs a warp about
-// 288 f32_ct FFMA issue slots and ~120 more of loads and bookkeeping, so wide items are the
-// efficient ones, but a stage runs in ceil(items / SMs) turns of an SM's four schedulers: the
-// shape of the least (turns x cost), wider ones first.
+// threads f32_groups x 8 pixels x 8, 16, 32 or 64 channels.  With n items per SM, a stage takes
+// max(alone, n x full) per chunk of input channels: `alone` is what a chunk takes while an SM
+// has fewer than about three items (its schedulers then wait for one or two warps' instruction
+// fetches and loads), `full` what it adds once they are busy.  Both in microseconds, measured on
+// GB300 with single layers of 38x38 to 152x152 (256 -> 512 3x3, 512 -> 256 1x1); e.g. 3x3 38x38:
+// 96 items of ct 8 took 355 us, 192 of ct 4 187, 384 of ct 2 123, 768 of ct 1 144; 152x152:
+// 1077, 1117, 1393 and 1754 us.
+struct F32Cost {
+    int ct;
+    double alone, full;
+};
+const F32Cost kF32Cost3[] = {{8, 5.5, 1.8}, {4, 2.9, 1.0}, {2, 1.9, 0.62}, {1, 1.5, 0.4}};
+const F32Cost kF32Cost1[] = {{8, 2.5, 1.2}, {4, 1.7, 0.6}, {2, 1.2, 0.47}, {1, 0.8, 0.31}};
+
 void f32_shape(MafatStageDev& s, const Layer& L, const std::vector<TileInfo>& tiles, int l, const PlanConfig& cfg,
                int n_ctas, PlanTables& t) {
     s.f32_rect = cfg.rect_blocks ? 1 : 0;
     double best = 0.0;
     int best_ct = 0;
-    for (int ct : {8, 4, 2, 1}) {
+    for (const F32Cost& fc : L.k == 3 ? kF32Cost3 : kF32Cost1) {
+        const int ct = fc.ct;
         MafatStageDev q = s;
         q.f32_groups = ct == 1 ? 8 : 16;
         const int nb = ct == 1 ? 16 : 8 * ct;
@@ -285,7 +296,7 @@ void f32_shape(MafatStageDev& s, const Layer& L, const std::vector<TileInfo>& ti
             if (!r.empty()) items += f32_region_items(q, r.h(), r.w());
         }
         items *= ceil_div(L.c_out, nb);
-        const double cost = (double)((items + n_ctas - 1) / n_ctas) * (288.0 * ct + 120.0);
+        const double cost = std::max(fc.alone, (double)items / n_ctas * fc.full);
         if (best_ct == 0 || cost < best) {
             best = cost;
             best_ct = ct;
