@@ -192,17 +192,26 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, uint32_
 // timeout is recorded by every lane alike (no branch on the lane).  The lanes poll in
 // step, so the result needs no vote: a vote and a warp barrier after every wait cost the
 // first layer ~7 % of its MMA phase.
+// The limit is looked up only once the first try has failed: a wait that is over costs one
+// try, and the code is small (it is part of every MMA instance, and what the MMA warp runs
+// between items mostly waits for instruction fetches).
+__device__ __noinline__ void pipe_timeout(uint32_t* ctr, volatile int* broken) {
+    mafat_dev::record_status(ctr, MAFAT_DEV_PIPE);
+    *broken = 1;
+}
 __device__ __forceinline__ void mbar_wait_mma(uint32_t bar, uint32_t parity, uint32_t* ctr, int64_t limit_ns,
                                               volatile int* broken) {
-    const uint64_t lim = (uint64_t)(*broken ? 1000000LL : limit_ns);
     uint32_t ok;
     asm volatile(
-        "{\n\t.reg .pred P1, P2;\n\t.reg .u64 dl, t;\n\t"
+        "{\n\t.reg .pred P1, P2;\n\t.reg .u64 dl, t;\n\t.reg .b32 br;\n\t"
         "mov.u32 %0, 1;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
         "@P1 bra MW_DONE_%=;\n\t"
+        "ld.volatile.shared.b32 br, [%4];\n\t"
+        "setp.ne.b32 P2, br, 0;\n\t"
+        "selp.b64 t, 1000000, %3, P2;\n\t"
         "mov.u64 dl, %%globaltimer;\n\t"
-        "add.u64 dl, dl, %3;\n\t"
+        "add.u64 dl, dl, t;\n\t"
         "MW_POLL_%=:\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
         "@P1 bra MW_DONE_%=;\n\t"
@@ -212,12 +221,9 @@ __device__ __forceinline__ void mbar_wait_mma(uint32_t bar, uint32_t parity, uin
         "mov.u32 %0, 0;\n\t"
         "MW_DONE_%=:\n\t}"
         : "=r"(ok)
-        : "r"(bar), "r"(parity), "l"(lim)
+        : "r"(bar), "r"(parity), "l"(limit_ns), "r"(smem_u32(const_cast<int*>(broken)))
         : "memory");
-    if (ok == 0u) {  // every lane polled the same barrier in step: ok is warp-uniform
-        mafat_dev::record_status(ctr, MAFAT_DEV_PIPE);
-        *broken = 1;
-    }
+    if (ok == 0u) pipe_timeout(ctr, broken);  // every lane polled the same barrier in step: ok is warp-uniform
 }
 
 // An arrive on bar by the lane with el = 1 (from elect_one).
@@ -642,6 +648,17 @@ __device__ __forceinline__ void mma_begin_piece(MmaState& s, MmaJob& j) {
     j.cur_b = b;
 }
 
+// The next piece of a streamed set: neither buffer holds a resident set any more.
+__device__ __forceinline__ void mma_next_piece(MmaState& s, MmaJob& j) {
+    const int b = s.wb.next;
+    s.wb.next ^= 1;
+    mbar_wait_mma(s.bar(kBarBFull + b), s.wb.loads(b) & 1u, s.ctr, s.pipe_limit, s.broken);
+    s.wb.loads0 += b ? 0u : 1u;
+    s.wb.loads1 += b ? 1u : 0u;
+    tc_fence_after();
+    j.cur_b = b;
+}
+
 // Low word of the B descriptor of the first blob of buffer b (start address in bits 0-13;
 // a later blob of the buffer only adds its offset >> 4 to it).
 __device__ __forceinline__ uint32_t b_lo_of(const MmaState& s, const MmaJob& j, int b) {
@@ -669,6 +686,7 @@ __device__ __forceinline__ void mma_item(MmaState& s, MmaJob& j) {
     uint32_t b_lo = b_lo_of(s, j, j.cur_b);
     const uint32_t blob16 = j.blob_bytes >> 4;
     const int taps = j.k * j.k;
+#pragma unroll 1
     for (int c = 0; c < j.n_chunks; ++c) {
         const int as = (int)(s.a_cnt % kAStages);
         const uint64_t tw0 = (TR && s.trace) ? mafat_dev::globaltimer_ns() : 0;
@@ -691,6 +709,7 @@ __device__ __forceinline__ void mma_item(MmaState& s, MmaJob& j) {
         const uint32_t a_base16 = (a_base & 0x3FFFFu) >> 4;
         uint32_t oa16 = 0, or16 = 0;
         int xa = 0;
+#pragma unroll 1
         for (int t = 0; t < j.n_bsteps; ++t) {
             uint32_t a_lo_t, a_hi_t;
             if (PAIRED) {
@@ -751,7 +770,7 @@ __device__ __forceinline__ void mma_item(MmaState& s, MmaJob& j) {
                 if (j.P > 1) tc_commit_el(s.el, s.bar(kBarBEmpty + j.cur_b));
                 if (g < j.G && t + 1 < j.n_bsteps) {
                     const uint64_t tp0 = (TR && s.trace) ? mafat_dev::globaltimer_ns() : 0;
-                    mma_begin_piece(s, j);
+                    mma_next_piece(s, j);
                     if (TR && s.trace) j.wait_b += mafat_dev::globaltimer_ns() - tp0;
                     rem = min(j.bpp, j.G - g);
                     b_lo = b_lo_of(s, j, j.cur_b);
@@ -762,7 +781,7 @@ __device__ __forceinline__ void mma_item(MmaState& s, MmaJob& j) {
         ++s.a_cnt;
         if (rem == 0 && g < j.G) {
             const uint64_t tp0 = (TR && s.trace) ? mafat_dev::globaltimer_ns() : 0;
-            mma_begin_piece(s, j);
+            mma_next_piece(s, j);
             if (TR && s.trace) j.wait_b += mafat_dev::globaltimer_ns() - tp0;
             rem = min(j.bpp, j.G - g);
             b_lo = b_lo_of(s, j, j.cur_b);
@@ -1216,6 +1235,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
                 if (j.cur_b < 0) mma_begin_piece(ms, j);
+                if (j.P > 1) ms.wb.key0 = ms.wb.key1 = -1;  // its pieces go through both buffers
                 const int buf = (int)(acc_cnt & 1u);
                 mbar_wait_mma(ms.bar(kBarAccEmpty + buf), ((acc_cnt >> 1) & 1u) ^ 1u, p.ctr, pipe_limit, broken);
                 tc_fence_after();
@@ -1261,8 +1281,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     MAFAT_MMA_CASE(1, 1, 5) MAFAT_MMA_CASE(1, 1, 6) MAFAT_MMA_CASE(1, 1, 7) MAFAT_MMA_CASE(1, 1, 8)
 #undef MAFAT_MMA_CASE
                     default:  // a shape the planner never makes: fail loudly, never compute silently wrong
-                        mafat_dev::record_status(p.ctr, MAFAT_DEV_PIPE);
-                        *broken = 1;
+                        pipe_timeout(p.ctr, broken);
                         break;
                 }
                 issued = true;
