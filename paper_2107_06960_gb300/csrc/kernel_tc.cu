@@ -167,9 +167,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 // net the first one to run out records MAFAT_DEV_PIPE and marks the CTA broken,
 // after which every pipeline wait of the CTA gives up after 1 ms, so the launch
 // still ends in bounded time (with garbage results and an error status).
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, uint32_t* ctr, int64_t limit_ns,
-                                          volatile int* broken, uint32_t sleep_ns = 0) {
-    if (mbar_try_wait(bar, parity)) return;
+// The polling loop and the give-up path are out of line, one copy for all waits.
+__device__ __noinline__ void pipe_timeout(uint32_t* ctr, volatile int* broken) {
+    mafat_dev::record_status(ctr, MAFAT_DEV_PIPE);
+    *broken = 1;
+}
+__device__ __noinline__ void mbar_poll(uint32_t bar, uint32_t parity, uint32_t* ctr, int64_t limit_ns,
+                                       volatile int* broken, uint32_t sleep_ns) {
     const int64_t lim = *broken ? 1000000LL : limit_ns;
     uint64_t t0 = mafat_dev::globaltimer_ns();
     for (uint32_t i = 1;; ++i) {
@@ -178,11 +182,14 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, uint32_
         if (sleep_ns) __nanosleep(sleep_ns);
         if (mbar_try_wait(bar, parity)) return;
         if ((i & 255u) == 0u && (int64_t)(mafat_dev::globaltimer_ns() - t0) > lim) {
-            mafat_dev::record_status(ctr, MAFAT_DEV_PIPE);
-            *broken = 1;
+            pipe_timeout(ctr, broken);
             return;
         }
     }
+}
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, uint32_t* ctr, int64_t limit_ns,
+                                          volatile int* broken, uint32_t sleep_ns = 0) {
+    if (!mbar_try_wait(bar, parity)) mbar_poll(bar, parity, ctr, limit_ns, broken, sleep_ns);
 }
 
 // The MMA warp's wait.  Measured on GB300: a polling loop written in C++ anywhere in
@@ -195,10 +202,6 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, uint32_
 // The limit is looked up only once the first try has failed: a wait that is over costs one
 // try, and the code is small (it is part of every MMA instance, and what the MMA warp runs
 // between items mostly waits for instruction fetches).
-__device__ __noinline__ void pipe_timeout(uint32_t* ctr, volatile int* broken) {
-    mafat_dev::record_status(ctr, MAFAT_DEV_PIPE);
-    *broken = 1;
-}
 __device__ __forceinline__ void mbar_wait_mma(uint32_t bar, uint32_t parity, uint32_t* ctr, int64_t limit_ns,
                                               volatile int* broken) {
     uint32_t ok;
