@@ -1105,6 +1105,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (trace && lane == 0) mafat_dev::trace_put(trace, ticket, 1, mafat_dev::globaltimer_ns());
                 if (ld.lookahead == 2) mbar_arrive_el(el, bar(kBarTake));
                 int next_pc = 1;  // the next weight piece to load (piece 0 went first)
+#pragma unroll 1
                 for (int c = 0; c < n_chunks; ++c) {
                     const int as = (int)(a_cnt % kAStages);
                     const uint32_t a_dst = sbase + kOffA + as * kAStageBytes;
@@ -1133,6 +1134,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     // the pieces that start inside this chunk (piece pc starts at blob pc * bpp);
                     // no division: on this single thread, a runtime modulo per blob cost ~1.5 us
                     // per chunk of a 3x3 256->512 item
+#pragma unroll 1
                     while (next_pc < P && next_pc * bpp < (c + 1) * n_bsteps) {
                         MAFAT_LOAD_PIECE(next_pc);
                         ++next_pc;

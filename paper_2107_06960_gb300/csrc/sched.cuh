@@ -43,22 +43,26 @@ __device__ __forceinline__ bool aborted(const uint32_t* ctr) {
     return *(volatile const uint32_t*)&ctr[MAFAT_CTR_ABORT] != 0u;
 }
 
-// Wait until ctr[idx] >= target (acquire), bounded by timeout_ns.
-__device__ __forceinline__ void wait_counter(uint32_t* ctr, int idx, int target, int64_t timeout_ns) {
-    if (idx < 0) return;
-    const uint32_t* p = ctr + idx;
-    if (ld_acquire_u32(p) >= (uint32_t)target) return;
-    // A poll is a round trip to L2 (~0.6 us), so a completion is seen about half of one late; the
-    // abort word, another round trip, is looked at every 16 polls.
+// Wait until ctr[idx] >= target (acquire), bounded by timeout_ns.  The polling loop is out of line:
+// the callers' code stays small, and what they run between items waits for instruction fetches.
+// A poll is a round trip to L2 (~0.6 us), so a completion is seen about half of one late; the
+// abort word, another round trip, is looked at every 16 polls.
+static __device__ __noinline__ void poll_counter(uint32_t* ctr, const uint32_t* p, uint32_t target, int64_t timeout_ns) {
     uint64_t t0 = globaltimer_ns();
+#pragma unroll 1
     for (uint32_t i = 1;; ++i) {
-        if (ld_acquire_u32(p) >= (uint32_t)target) return;
+        if (ld_acquire_u32(p) >= target) return;
         if ((i & 15u) == 0u && aborted(ctr)) return;
         if ((int64_t)(globaltimer_ns() - t0) > timeout_ns) {
             record_status(ctr, MAFAT_DEV_TIMEOUT);
             return;
         }
     }
+}
+__device__ __forceinline__ void wait_counter(uint32_t* ctr, int idx, int target, int64_t timeout_ns) {
+    if (idx < 0) return;
+    const uint32_t* p = ctr + idx;
+    if (ld_acquire_u32(p) < (uint32_t)target) poll_counter(ctr, p, (uint32_t)target, timeout_ns);
 }
 
 __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
