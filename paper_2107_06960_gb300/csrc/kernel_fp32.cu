@@ -20,14 +20,15 @@
 // neighbouring groups of one warp (one exchange), neighbouring pixels are in one thread.
 //
 // Which CT (8, 4, 2, or 1 with half the groups) a stage runs is the planner's choice
-// (f32_shape): large stages take CT = 8, which is nearest the FFMA rate; stages with less
-// than a wave of such items take narrower ones, which spread over more SMs.
+// (f32_shape): large stages take CT = 8, which is nearest the FFMA rate; stages with fewer
+// than about three such items per SM take narrower ones, which spread over more warps.
 //
 // Measured on GB300: a 3x3 128 -> 256 convolution of 152x152 at 50 TFLOP/s (0.27 ms; a thread
 // per pixel reading both operands from L1 took ~30 times as long), 1x1 256 -> 128 at 25; the
-// 16-layer network at 416x416 29.06 -> 1.04 ms, two 96x96 frames 53.9 -> 0.55 ms.  Those small
-// frames are bound by their chain of 26 dependent layers (10-35 us each: a 64-chunk item of one
-// warp per scheduler takes 0.5 us a chunk).  Measured and not kept: the halo held twice in shared
+// 16-layer network at 416x416 29.06 -> 0.83 ms, two 96x96 frames 53.9 -> 0.30 ms (the shapes'
+// choice and, for the two frames, the hand-out order included).  Those small frames are bound by
+// their chain of 13 dependent layers (10-45 us each: a 64-chunk item of one warp per scheduler
+// takes ~0.7 us a chunk).  Measured and not kept: the halo held twice in shared
 // memory so that pair instructions need no moves (42 instead of 50 TFLOP/s: 30 % more loads);
 // a chunk's rows unrolled (a lone warp's instruction fetches); 128 registers and 4 CTAs per SM.
 #include "sched.cuh"

@@ -2,6 +2,14 @@
 // (MAFAT, Sec. 3-4) on sm_103a: tcgen05 MMA with TMEM accumulators, operands
 // staged in shared memory by TMA, one persistent launch per plan.
 //
+// The kernel is bound by the chain of dependent layers (one frame) and by what its warps do between
+// items (many frames), not by DRAM (2 % of its bandwidth) or the tensor core: every role is a warp
+// or two on a scheduler of its own, and such a warp mostly waits for its instructions.  So the
+// roles' loops are converged, small and nearly free of branches: arrivals, copies and stores are
+// predicated in asm, loops are not unrolled, polling and failure paths are out of line.  Measured
+// on GB300 from the form before (one thread for tickets, records and loads; lane branches; 231 KB
+// of code, now 144): 608x608 93.8 -> 79 us, 16 frames 1009 -> 678, 8 1216x1216 frames 1478 -> 1142.
+//
 // One work item = up to 8 vertically stacked 16 x 8 blocks of a tile's conv
 // output (M = 128 pixels each, one accumulator each) times one block of n_blk
 // <= 256 output channels, i.e. an implicit GEMM
@@ -23,7 +31,7 @@
 //  * B: weights pre-packed on the host in exactly their shared-memory image, as
 //    blobs of one (chunk, tap); blobs with 64 channels use the 128-byte swizzled
 //    K-major layout, narrower ones the no-swizzle one.  The weights of one (stage,
-//    output-channel block) travel in pieces filling one of two 74 KB buffers: a
+//    output-channel block) travel in pieces filling one of two 73 KB buffers: a
 //    set that fits one piece stays resident while the CTA's consecutive items use
 //    it, larger sets stream piece by piece (every copy costs a few hundred cycles
 //    of TMA time however small it is, so copies are large and few).
@@ -562,7 +570,7 @@ __device__ __forceinline__ float max_f32(uint32_t a, uint32_t b) {
     return fmaxf(__uint_as_float(a), __uint_as_float(b));
 }
 
-// Weight-buffer bookkeeping.  The producer and the MMA issuer each keep a copy and
+// Weight-buffer bookkeeping.  The loader and the MMA issuer each keep a copy and
 // apply the same transitions to the same item sequence, so they agree without
 // talking on which of the two buffers holds which weights.  A set that fits one
 // piece stays resident in its buffer (key >= 0) across items that use it; larger
@@ -769,7 +777,7 @@ __device__ __forceinline__ void mma_item(MmaState& s, MmaJob& j) {
                 // end of the buffer's blobs for this item: a streamed piece is released as soon
                 // as its last blob has been issued, and the next piece (if any) is waited for;
                 // a piece that ends with the chunk is followed only after the A stage is
-                // released below, so that the producer can refill the stage meanwhile
+                // released below, so that the loader can refill the stage meanwhile
                 if (j.P > 1) tc_commit_el(s.el, s.bar(kBarBEmpty + j.cur_b));
                 if (g < j.G && t + 1 < j.n_bsteps) {
                     const uint64_t tp0 = (TR && s.trace) ? mafat_dev::globaltimer_ns() : 0;
@@ -1232,7 +1240,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (j.P > 1) {
                     // a streamed set takes both buffers: a resident set held in the one its
                     // second piece goes to is released now (its MMAs are long done), not when
-                    // that piece is needed, so that the producer can load the piece meanwhile
+                    // that piece is needed, so that the loader can load the piece meanwhile
                     const int o = ms.wb.next ^ 1;
                     if (ms.wb.held(o)) {
                         tc_commit_el(ms.el, ms.bar(kBarBEmpty + o));
@@ -1364,11 +1372,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (warp == kGatherWarp) {
         // ------------------------------------------------------------ gather warp (warp 11)
         // For items whose input is a narrow NHWC image (fewer than 8 channels, e.g. RGB), the
-        // producer lands raw rows of the image in the A stage's tail; this warp expands them
+        // loader lands raw rows of the image in the A stage's tail; this warp expands them
         // into the one-octet halo the MMAs read ([rows][cols][8 channels], channels c..7
         // zero), makes the stores visible to the tensor core (async proxy) and completes the
         // stage's full barrier.  It walks the item queue like the other consumers, counting A
-        // stages as the producer and the MMA warp do.
+        // stages as the loader and the MMA warp do.
         uint32_t q_cnt = 0, a_cnt = 0, raw_uses0 = 0, raw_uses1 = 0;
         while (true) {
             const int qs = (int)(q_cnt % kQDepth);
