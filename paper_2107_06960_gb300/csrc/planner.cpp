@@ -645,12 +645,24 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
     // Several frames with a ring each, where that stays small, so that a frame's first tiles need
     // not wait for the last stages of the frame before: a frame's chain of layers is longer than
     // the time its work keeps the SMs busy.  The limit keeps the rings in the 129 MB L2; an fp32
-    // plan's also leave room in the 32 MiB area of the allocation-free call.
+    // plan's also in the 32 MiB area of the allocation-free call, next to the cut tensor, the outputs
+    // of the groups between and the counters, so that more rings never push a plan out of it.
     const bool reorder = cfg.batch > 1 && !cfg.halo_reuse && !cfg.frame_major && cfg.ring_slots <= 0 && cfg.wave_tiles <= 0 &&
                          W >= max_tiles && S >= tiles_per_frame;
     if (reorder && cfg.batch > 1 && S == tiles_per_frame) {
         const int64_t set_bytes = (int64_t)S * 2 * t.slot_buf_elems * (cfg.dtype == 0 ? 2 : 4);
-        const int64_t limit = cfg.dtype == 0 ? (int64_t)112 << 20 : (int64_t)16 << 20;
+        int64_t limit = (int64_t)112 << 20;
+        if (cfg.dtype != 0) {
+            int64_t others = G > 1 ? cut_frame * cfg.batch : 0;  // 4-byte elements and counters
+            for (int g = 0; g < G; ++g) {
+                const MafatStageDev& st = t.stages[t.stage_last[g]];
+                const Layer& Lo = net.layers[t.groups[g][1]];
+                if (g > 0 && g + 1 < G)
+                    others += (int64_t)ceil_div(st.cout, 8) * 8 * Lo.h_out * Lo.w_out * cfg.batch + 128;
+                others += ((int64_t)tiles[g].size() * (t.stage_last[g] - t.stage_first[g] + 1) + 1) * cfg.batch;
+            }
+            limit = std::min<int64_t>((int64_t)16 << 20, ((int64_t)32 << 20) - others * 4 - 4096);
+        }
         t.ring_sets = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(cfg.batch, 4), limit / std::max<int64_t>(set_bytes, 1)));
     }
     const int S_all = S * t.ring_sets;
