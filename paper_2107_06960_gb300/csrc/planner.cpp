@@ -633,14 +633,19 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
 
     // ---- scratch buffer size: largest non-final stage output of any tile
     int64_t buf = 0;
+    std::vector<int64_t> tile_buf;  // the same of each tile of a frame, in the order of the tiles
     for (int g = 0; g < G; ++g)
-        for (const TileInfo& ti : tiles[g])
+        for (const TileInfo& ti : tiles[g]) {
+            int64_t b = 0;
             for (int s = t.stage_first[g]; s < t.stage_last[g]; ++s) {
                 const MafatStageDev& st = t.stages[s];
                 int ol = stage_pool_layer[s] >= 0 ? stage_pool_layer[s] : st.layer;
                 const Rect& r = ti.outs[ol];
-                buf = std::max(buf, (int64_t)r.h() * r.w() * ceil_div(st.cout, 8) * 8);
+                b = std::max(b, (int64_t)r.h() * r.w() * ceil_div(st.cout, 8) * 8);
             }
+            buf = std::max(buf, b);
+            tile_buf.push_back((b + 127) / 128 * 128);
+        }
     t.slot_buf_elems = (buf + 127) / 128 * 128;  // 256-byte aligned for bf16, 512 for fp32
     // Several frames with a ring each, where that stays small, so that a frame's first tiles need
     // not wait for the last stages of the frame before: a frame's chain of layers is longer than
@@ -649,8 +654,18 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
     // of the groups between and the counters, so that more rings never push a plan out of it.
     const bool reorder = cfg.batch > 1 && !cfg.halo_reuse && !cfg.frame_major && cfg.ring_slots <= 0 && cfg.wave_tiles <= 0 &&
                          W >= max_tiles && S >= tiles_per_frame;
-    if (reorder && cfg.batch > 1 && S == tiles_per_frame) {
-        const int64_t set_bytes = (int64_t)S * 2 * t.slot_buf_elems * (cfg.dtype == 0 ? 2 : 4);
+    // A ring of a whole frame gives each tile a slot of its own: a bf16 plan's slots are then as large
+    // as their tiles need (608x608, 5x5 / 2x2: 22.7 MB a ring instead of 54.9, whose slots all held a
+    // second-group tile), so that more rings fit: four such frames 204 -> 170 us.  fp32 rings stay as
+    // they were, so that the allocation-free call takes the plans that it took and no others.
+    const bool own_slots = reorder && S == tiles_per_frame && cfg.dtype == 0;
+    if (reorder && S == tiles_per_frame) {
+        int64_t set_elems = (int64_t)S * 2 * t.slot_buf_elems;
+        if (own_slots) {
+            set_elems = 0;
+            for (int64_t b : tile_buf) set_elems += 2 * b;
+        }
+        const int64_t set_bytes = set_elems * (cfg.dtype == 0 ? 2 : 4);
         int64_t limit = (int64_t)112 << 20;
         if (cfg.dtype != 0) {
             int64_t others = G > 1 ? cut_frame * cfg.batch : 0;  // 4-byte elements and counters
@@ -666,7 +681,12 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
         t.ring_sets = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(cfg.batch, 4), limit / std::max<int64_t>(set_bytes, 1)));
     }
     const int S_all = S * t.ring_sets;
-    t.scratch_elems = (int64_t)S_all * 2 * t.slot_buf_elems;
+    t.slot_off.assign(1, 0);
+    for (int i = 0; i < S_all; ++i) t.slot_off.push_back(t.slot_off[i] + 2 * (own_slots ? tile_buf[i % S] : t.slot_buf_elems));
+    t.scratch_elems = t.slot_off[S_all];
+    auto slot_buf = [&](int slot, int half) {  // offset of one of a slot's two buffers
+        return t.slot_off[slot] + half * ((t.slot_off[slot + 1] - t.slot_off[slot]) / 2);
+    };
     // halo reuse: one whole output map per non-final stage, every frame, instead of the ring
     std::vector<int64_t> map_off(t.stages.size(), -1), map_frame(t.stages.size(), 0);
     std::vector<int> map_h(t.stages.size(), 0), map_w(t.stages.size(), 0), stage_tmap(t.stages.size(), -1);
@@ -795,16 +815,16 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                             tk.in_x0 = 0;
                             tk.in_tmap = stage_tmap[s];
                         } else {
-                            int b = (slot * 2) + ((rel - 1) & 1);
+                            const int64_t b = slot_buf(slot, (rel - 1) & 1);
                             tk.in_kind = MAFAT_BUF_SCRATCH;
-                            tk.in_off = (int64_t)b * t.slot_buf_elems;
+                            tk.in_off = b;
                             tk.in_h = ir.h();
                             tk.in_w = ir.w();
                             tk.in_y0 = ir.y0;
                             tk.in_x0 = ir.x0;
                             TmapReq req{};
                             req.task = (int)t.tasks.size();
-                            req.elem_off = (int64_t)b * t.slot_buf_elems;
+                            req.elem_off = b;
                             req.frames = 1;
                             req.h = ir.h();
                             req.w = ir.w();
@@ -846,10 +866,9 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                             tk.out_y0 = 0;
                             tk.out_x0 = 0;
                         } else {
-                            int b = (slot * 2) + (rel & 1);
                             tk.out_kind = MAFAT_BUF_SCRATCH;
                             tk.out_nhwc = 0;
-                            tk.out_off = (int64_t)b * t.slot_buf_elems;
+                            tk.out_off = slot_buf(slot, rel & 1);
                             tk.out_h = orr.h();
                             tk.out_w = orr.w();
                             tk.out_y0 = orr.y0;
@@ -1093,7 +1112,15 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
     const int64_t cut_total = (int64_t)t.cfg.batch * t.cut_c8 * 8 * t.cut_h * t.cut_w;
     const int64_t out_total = (int64_t)t.cfg.batch * t.out_h * t.out_w * t.out_c;
     const int64_t scratch_total = t.scratch_elems;
-    if (!t.cfg.halo_reuse && scratch_total < (int64_t)t.ring_slots * t.ring_sets * 2 * t.slot_buf_elems) return "scratch below the ring";
+    if (!t.cfg.halo_reuse && ((int64_t)t.slot_off.size() != (int64_t)t.ring_slots * t.ring_sets + 1 || scratch_total < t.slot_off.back()))
+        return "scratch below the ring";
+    // elements from a ring offset to the end of its buffer, 0 where no buffer starts there
+    auto ring_buf = [&](int64_t off) -> int64_t {
+        const size_t i = std::upper_bound(t.slot_off.begin(), t.slot_off.end(), off) - t.slot_off.begin();
+        if (i == 0 || i >= t.slot_off.size()) return 0;
+        const int64_t half = (t.slot_off[i] - t.slot_off[i - 1]) / 2, at = off - t.slot_off[i - 1];
+        return at == 0 || at == half ? half : 0;
+    };
     auto buf_total = [&](int kind) {
         return kind == MAFAT_BUF_USER_IN ? in_total
                : kind == MAFAT_BUF_CUT   ? cut_total
@@ -1206,7 +1233,8 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
             return "input region does not cover the conv rectangle's taps";
         if (k.in_y0 + k.in_h > L.h_in || k.in_x0 + k.in_w > L.w_in || k.in_y0 < 0 || k.in_x0 < 0)
             return "input region outside the map";
-        if (k.in_kind == MAFAT_BUF_SCRATCH && k.in_off % t.slot_buf_elems != 0) return "scratch input misaligned";
+        if (k.in_kind == MAFAT_BUF_SCRATCH && (int64_t)((L.c_in + 7) / 8) * 8 * k.in_h * k.in_w > ring_buf(k.in_off))
+            return "scratch input outside its buffer";
         if (k.dep_count < 0 || k.dep_first < 0 || k.dep_first + k.dep_count > (int)t.deps.size()) return "bad dependency list";
         for (int d = k.dep_first; d < k.dep_first + k.dep_count; ++d) {
             const int dt = t.deps[d].ctr - MAFAT_CTR_BASE;
@@ -1226,7 +1254,7 @@ std::string validate_plan(const Net& net, const PlanTables& t) {
                                        : (int64_t)((so.cout + 7) / 8) * 8 * k.out_h * k.out_w;
         if (k.out_off < 0 || k.out_off + out_elems > buf_total(k.out_kind)) return "output buffer outside its allocation";
         if (out_elems >= ((int64_t)1 << 31)) return "an output region exceeds 2^31 elements";
-        if (k.out_kind == MAFAT_BUF_SCRATCH && out_elems > t.slot_buf_elems) return "scratch output above buffer size";
+        if (k.out_kind == MAFAT_BUF_SCRATCH && out_elems > ring_buf(k.out_off)) return "scratch output above buffer size";
         if (k.done_ctr < MAFAT_CTR_BASE || k.done_ctr >= MAFAT_CTR_BASE + t.n_counters) return "bad done counter";
     }
     // dependencies: every counter an item waits on is fed only by items handed out before it

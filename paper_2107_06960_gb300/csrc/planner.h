@@ -121,7 +121,8 @@ struct PlanTables {
     int64_t weight32_elems = 0;          // fp32 weight elements
     int64_t pack32_elems = 0;            // fp32 weights as packed for the kernel (with padding)
     int64_t sb_elems = 0;                // scale / bias elements
-    int64_t slot_buf_elems = 0;          // elements of one ping-pong buffer
+    int64_t slot_buf_elems = 0;          // elements of the largest ping-pong buffer
+    std::vector<int64_t> slot_off;       // offset of each ring slot's two buffers, then the ring's end
     int64_t scratch_elems = 0;           // the scratch allocation (ring, or layer maps with halo reuse)
     std::vector<MafatDepDev> deps;       // task dependency lists (halo reuse)
     int ring_slots = 0, wave_tiles = 0;
