@@ -60,7 +60,7 @@ typedef enum { MAFAT_CONV = 0, MAFAT_MAXPOOL = 1 } mafat_layer_type;
 
 /* Arithmetic of a plan.  BF16: bf16 activations and weights, fp32 accumulation
  * on the tensor cores (tcgen05), every layer output rounded to bf16.  FP32: the
- * same fused tiling computed in fp32 on the CUDA cores (a check mode). */
+ * same fused tiling computed in fp32 on the CUDA cores. */
 typedef enum { MAFAT_BF16 = 0, MAFAT_FP32 = 1 } mafat_dtype;
 
 /* One layer of the network description (the W, H, F, S vectors of Sec. 4.1 and
@@ -81,7 +81,8 @@ typedef struct mafat_plan_s mafat_plan_t;
 /* Optional knobs of mafat_plan_ex.  Zero-initialise and set struct_size. */
 typedef struct {
     int32_t struct_size;        /* sizeof(mafat_plan_options) */
-    int32_t ring_slots;         /* tiles whose intermediate buffers may be live at once (0: default) */
+    int32_t ring_slots;         /* tiles whose intermediate buffers may be live at once (0: chosen; a
+                                   batch > 1 may then hold up to four rings of one frame's tiles each) */
     int32_t wave_tiles;         /* tiles whose layers are interleaved in the work order (0: = ring_slots) */
     int32_t max_ctas;           /* persistent CTAs (0: one per SM) */
     int64_t wait_timeout_ns;    /* limit of a device-side wait before MAFAT_ETIMEOUT (0: 2 s) */
@@ -105,9 +106,10 @@ typedef struct {
                                    and reads the halo its next layer needs from its neighbours' parts
                                    (each layer waits for those neighbours); 0: the fused tiles of
                                    Sec. 3-4, every tile recomputing its halo */
-    int32_t frame_major;        /* batch > 1 with two groups: 1 hands the frames out strictly one after
-                                   another; 0 (default) overlaps frame f's second group with frame
-                                   f + 1's first (the second group's small maps leave SMs idle) */
+    int32_t frame_major;        /* batch > 1: 1 hands the frames out strictly one after another; 0
+                                   (default) overlaps them where that is expected to be faster (small
+                                   maps leave SMs idle), e.g. frame f's second group with frame f + 1's
+                                   first */
     int32_t chain;              /* BF16 plans: 1 chains a 3x3 convolution and the 1x1 convolution after
                                    it inside one work item where both fit one TMEM accumulator buffer:
                                    the 3x3's activated bf16 output stays in tensor memory and is the

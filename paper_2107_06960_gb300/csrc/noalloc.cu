@@ -5,7 +5,7 @@
 // global mode (cudaMalloc is refused there), real-time loops that forbid
 // allocator calls, or host processes whose device memory is owned by another
 // allocator and budgeted up front.  mafat_run_fp32_noalloc serves them: it runs
-// the fp32 check kernel of an already-created plan, taking every byte of
+// the fp32 kernel of an already-created plan, taking every byte of
 // per-run scratch (the ring of tile buffers, the cut tensor between the two
 // layer groups, and the scheduler counters) from one fixed device array that
 // is part of this library, instead of from the plan's own workspace.  It makes
