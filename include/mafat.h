@@ -284,7 +284,8 @@ mafat_status mafat_search(const mafat_net_t* net, double limit_mib, double bias_
  * device; here the memory that matters is the L2 that a plan's intermediates (tile
  * scratch ring and cut tensor) should stay in, and latency is measured rather than
  * predicted: every candidate within budget_bytes is planned and timed on the device,
- * and the fastest is reported.  Candidates, in this order: one layer group (if
+ * and the fastest is reported.  The plan sized and timed is the one that mafat_plan
+ * makes of the candidate (with the ring_slots that it names).  Candidates, in this order: one layer group (if
  * include_one_group), then two groups at each cut of cuts[0..n_cuts-1] (the first
  * layer of group 2), every group tiled N x M for N, M in 1..max_grid (N == M when
  * square_only, else |N - M| <= 1), group 1's tiling outer. */
@@ -308,12 +309,14 @@ typedef struct {
 typedef struct {
     int32_t n_groups, cut;      /* cut is 0 for one group */
     int32_t grid_n[2], grid_m[2];
-    int64_t intermediate_bytes; /* tile scratch ring + cut tensor of the plan */
+    int64_t intermediate_bytes; /* tile scratch rings + cut tensor of the plan */
     double predicted_mib;       /* Algorithm 1 (literal reading, 31 MiB bias) for the configuration */
     double executed_flops;      /* per run, halo recompute included */
     double us_per_run;          /* median device time of a run; < 0 if not timed */
     int32_t status;             /* MAFAT_OK if timed; MAFAT_ENOFIT over budget; else the plan's error */
-    int32_t reserved;
+    int32_t ring_slots;         /* mafat_plan_options.ring_slots of the plan that was sized and timed: 0 (the
+                                   default plan), or one ring of tiles where a batch > 1 is over the budget
+                                   with the rings that the default plan holds */
 } mafat_search_candidate;
 
 /* Runs the measured search on `stream` (the net's weights must be set; the input is

@@ -58,7 +58,7 @@ class SearchOptions(ctypes.Structure):
 class SearchCandidate(ctypes.Structure):
     _fields_ = [("n_groups", i32), ("cut", i32), ("grid_n", i32 * 2), ("grid_m", i32 * 2),
                 ("intermediate_bytes", i64), ("predicted_mib", dbl), ("executed_flops", dbl),
-                ("us_per_run", dbl), ("status", i32), ("reserved", i32)]
+                ("us_per_run", dbl), ("status", i32), ("ring_slots", i32)]
 
 
 # (name, restype, argtypes) of every entry point of include/mafat.h
@@ -211,8 +211,8 @@ class Net:
                         budget_bytes=0, runs=10, flush_l2=True, dry_run=False, batch=1, dtype=BF16, stream=None):
         """Measured plan search (mafat_search_measured): returns (candidates, best index), each
         candidate a dict with n_groups, cut (None for one group), grids [(n, m), ...],
-        intermediate_bytes, predicted_mib, executed_flops, us_per_run (None if not timed) and
-        status."""
+        intermediate_bytes, predicted_mib, executed_flops, us_per_run (None if not timed), status
+        and ring_slots (pass it to Plan, with the cut and grids, for the plan that was timed)."""
         opt = SearchOptions()
         opt.struct_size = ctypes.sizeof(SearchOptions)
         opt.batch, opt.dtype, opt.include_one_group = batch, dtype, int(include_one_group)
@@ -232,7 +232,8 @@ class Net:
                         "grids": [(c.grid_n[i], c.grid_m[i]) for i in range(g)],
                         "intermediate_bytes": c.intermediate_bytes, "predicted_mib": c.predicted_mib,
                         "executed_flops": c.executed_flops,
-                        "us_per_run": c.us_per_run if c.us_per_run >= 0 else None, "status": c.status})
+                        "us_per_run": c.us_per_run if c.us_per_run >= 0 else None, "status": c.status,
+                        "ring_slots": c.ring_slots})
         return res, best.value
 
     def close(self):

@@ -112,46 +112,46 @@ mafat_status mafat_search_measured(const mafat_net_t* net, const mafat_search_op
         r.us_per_run = -1.0;
         r.status = MAFAT_OK;
         const int32_t cut = c.cut;
+        int64_t cut_bytes = 0;
+        if (c.n_groups == 2) {
+            int32_t sh[6];
+            if (mafat_net_shape(net, c.cut - 1, sh) == MAFAT_OK)
+                cut_bytes = (int64_t)batch * ((sh[5] + 7) / 8) * 8 * sh[3] * sh[4] * (int64_t)esz;
+        }
+        // The plan that is sized is the one that is timed and that the caller gets: the default plan,
+        // or, where that is over the budget, the same configuration with one ring of tiles (a batched
+        // plan's further rings are only there for speed), which the candidate's ring_slots names.
         mafat_plan_options po{};
         po.struct_size = (int32_t)sizeof(po);
-        po.dry_run = 1;
+        po.test_unpublished_task = -1;
         mafat_plan_t* plan = nullptr;
-        st = mafat_plan_ex(net, c.n_groups, &cut, c.gn, c.gm, batch, opt->dtype, &po, &plan);
-        mafat_plan_options run_po{};
-        run_po.struct_size = (int32_t)sizeof(run_po);
-        run_po.test_unpublished_task = -1;
-        if (st == MAFAT_OK && batch > 1) {
-            // candidates are compared, and held to the budget, with one ring of tiles: the rings a
-            // batched plan adds where memory is plentiful would count against a budget that it fits
-            mafat_plan_stats_t ps{};
-            ps.struct_size = (int32_t)sizeof(ps);
-            mafat_plan_stats(plan, &ps);
-            mafat_plan_destroy(plan);
-            plan = nullptr;
-            po.ring_slots = run_po.ring_slots = ps.ring_slots;
+        for (int pass = 0; pass < 2; ++pass) {
+            po.dry_run = 1;
             st = mafat_plan_ex(net, c.n_groups, &cut, c.gn, c.gm, batch, opt->dtype, &po, &plan);
-        }
-        if (st == MAFAT_OK) {
+            if (st != MAFAT_OK) {
+                r.status = st;
+                break;
+            }
             mafat_plan_stats_t ps{};
             ps.struct_size = (int32_t)sizeof(ps);
             mafat_plan_stats(plan, &ps);
             mafat_plan_destroy(plan);
             plan = nullptr;
-            int64_t cut_bytes = 0;
-            if (c.n_groups == 2) {
-                int32_t sh[6];
-                if (mafat_net_shape(net, c.cut - 1, sh) == MAFAT_OK)
-                    cut_bytes = (int64_t)batch * ((sh[5] + 7) / 8) * 8 * sh[3] * sh[4] * (int64_t)esz;
+            po.dry_run = 0;
+            const int64_t bytes = ps.scratch_bytes + cut_bytes;
+            const bool fits = budget <= 0 || bytes <= budget;
+            if (pass == 0 || fits) {  // over the budget either way: refused with the default plan's size
+                r.intermediate_bytes = bytes;
+                r.predicted_mib = ps.predicted_mib;
+                r.executed_flops = ps.executed_flops;
+                r.ring_slots = po.ring_slots;
+                r.status = fits ? MAFAT_OK : MAFAT_ENOFIT;
             }
-            r.intermediate_bytes = ps.scratch_bytes + cut_bytes;
-            r.predicted_mib = ps.predicted_mib;
-            r.executed_flops = ps.executed_flops;
-            if (budget > 0 && r.intermediate_bytes > budget) r.status = MAFAT_ENOFIT;
-        } else {
-            r.status = st;
+            if (fits || batch == 1) break;
+            po.ring_slots = ps.ring_slots;
         }
         if (!dry && r.status == MAFAT_OK) {
-            st = mafat_plan_ex(net, c.n_groups, &cut, c.gn, c.gm, batch, opt->dtype, &run_po, &plan);
+            st = mafat_plan_ex(net, c.n_groups, &cut, c.gn, c.gm, batch, opt->dtype, &po, &plan);
             if (st != MAFAT_OK) {
                 r.status = st;
             } else {
