@@ -84,7 +84,8 @@ typedef struct {
     int32_t ring_slots;         /* tiles whose intermediate buffers may be live at once (0: chosen; a
                                    batch > 1 may then hold up to four rings of one frame's tiles each) */
     int32_t wave_tiles;         /* tiles whose layers are interleaved in the work order (0: = ring_slots) */
-    int32_t max_ctas;           /* persistent CTAs (0: one per SM) */
+    int32_t max_ctas;           /* persistent CTAs (0: BF16 one per SM, which is also the most a BF16 plan
+                                   takes; FP32 three per SM) */
     int64_t wait_timeout_ns;    /* limit of a device-side wait before MAFAT_ETIMEOUT (0: 2 s) */
     int32_t test_unpublished_task; /* test hook: index of a task whose completion is never
                                       published, so that waits on it run out (-1: none) */

@@ -394,6 +394,9 @@ mafat_status mafat_plan_ex(const mafat_net_t* net, int32_t n_groups, const int32
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     }
     if (sms <= 0) sms = 152;
+    // The tensor-core kernel hands its first items out by CTA index, so every CTA has to be resident
+    // from the start (sched.cuh): no more than one per SM, which is what an SM holds.
+    if (dt == MAFAT_BF16 && o.max_ctas > sms) o.max_ctas = sms;
     cfg.n_ctas = o.max_ctas > 0 ? o.max_ctas : sms;
 
     mafat_plan_s* p = new (std::nothrow) mafat_plan_s();

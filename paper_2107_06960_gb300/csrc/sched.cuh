@@ -4,7 +4,10 @@
 // dependency of an item (the previous fused stage of its tile, the tile that
 // last used its scratch slot, or all group-1 tiles of its frame) consists of
 // items with smaller tickets, and a CTA only takes a ticket while it runs, so
-// the smallest unfinished ticket can always make progress.  Waits are bounded
+// the smallest unfinished ticket can always make progress.  (The tensor-core
+// kernel's first gridDim.x tickets go out by CTA index, without the atomic's round
+// trip: its grid is never larger than the SMs, one CTA each, so that all of its
+// CTAs run from the start.)  Waits are bounded
 // by a wall-clock limit: when it runs out the kernel records
 // MAFAT_DEV_TIMEOUT, raises the abort word and every later wait returns at
 // once, so the launch always ends.
