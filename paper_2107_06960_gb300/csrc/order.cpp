@@ -113,6 +113,29 @@ struct Model {
     }
 };
 
+// The model of a plan; items: each stage's items of one frame.
+Model make_model(const PlanTables& t, const std::vector<TaskDep>& deps, std::vector<double>& items) {
+    Model m{t, deps, {}, t.cfg.dtype == 0, t.cfg.n_ctas > 0 ? t.cfg.n_ctas : 152};
+    std::vector<double> blocks(t.stages.size(), 0.0);
+    items.assign(t.stages.size(), 0.0);
+    for (const MafatTaskDev& k : t.tasks) {
+        if (k.frame != 0) continue;
+        blocks[k.stage] += (double)k.nby * k.nbx * t.stages[k.stage].n_nblk;
+        items[k.stage] += k.n_items;
+    }
+    for (size_t s = 0; s < t.stages.size(); ++s)
+        m.cost.push_back(m.tc ? tc_cost(t.stages[s], items[s] > 0 ? blocks[s] / items[s] : 1.0) : f32_cost(t.stages[s]));
+    return m;
+}
+
+// Modelled time of the tasks of the first frames, in the order given.
+double run_prefix(const Model& m, const std::vector<int>& order, int frames) {
+    std::vector<int> prefix;
+    for (int i : order)
+        if (m.t.tasks[i].frame < frames) prefix.push_back(i);
+    return m.run(prefix);
+}
+
 // Topological order of the tasks with smallest key first.
 std::vector<int> topological(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<double>& key,
                              int frames) {
@@ -146,30 +169,29 @@ std::vector<int> topological(const PlanTables& t, const std::vector<TaskDep>& de
 
 }  // namespace
 
+double modelled_us(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& order, int frames) {
+    std::vector<double> items;
+    return run_prefix(make_model(t, deps, items), order, frames);
+}
+
 std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& given) {
     const int G = t.cfg.n_groups, n = (int)t.tasks.size(), batch = t.cfg.batch;
-    Model m{t, deps, {}, t.cfg.dtype == 0, t.cfg.n_ctas > 0 ? t.cfg.n_ctas : 152};
+    std::vector<double> items;
+    const Model m = make_model(t, deps, items);
     const size_t n_st = t.stages.size();
-    std::vector<double> blocks(n_st, 0.0), items(n_st, 0.0);
     std::vector<int> tile(n, 0), tiles(n_st, 0);  // tile index of a task among its stage's of the frame
     int64_t frame_items = 0;
     for (int i = 0; i < n; ++i) {
-        const MafatTaskDev& k = t.tasks[i];
-        if (k.frame != 0) continue;
-        blocks[k.stage] += (double)k.nby * k.nbx * t.stages[k.stage].n_nblk;
-        items[k.stage] += k.n_items;
-        frame_items += k.n_items;
-        ++tiles[k.stage];
+        if (t.tasks[i].frame != 0) continue;
+        frame_items += t.tasks[i].n_items;
+        ++tiles[t.tasks[i].stage];
     }
     {
         std::vector<int> seen((size_t)batch * n_st, 0);
         for (int i = 0; i < n; ++i) tile[i] = seen[(size_t)t.tasks[i].frame * n_st + t.tasks[i].stage]++;
     }
     std::vector<double> work(n_st, 0.0);  // microseconds of all SMs for a stage of one frame
-    for (size_t s = 0; s < n_st; ++s) {
-        m.cost.push_back(m.tc ? tc_cost(t.stages[s], items[s] > 0 ? blocks[s] / items[s] : 1.0) : f32_cost(t.stages[s]));
-        work[s] = items[s] * m.cost[s].period / (m.tc ? m.n_ctas : 3 * m.n_ctas);
-    }
+    for (size_t s = 0; s < n_st; ++s) work[s] = items[s] * m.cost[s].period / (m.tc ? m.n_ctas : 3 * m.n_ctas);
     std::vector<double> gw(G, 0.0), off(n_st, 0.0);
     double total = 0.0;
     for (int g = 0; g < G; ++g) {
@@ -200,15 +222,9 @@ std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>&
         }
         return key;
     };
-    auto given_us = [&](int frames) {
-        std::vector<int> prefix;
-        for (int i : given)
-            if (t.tasks[i].frame < frames) prefix.push_back(i);
-        return m.run(prefix);
-    };
     // the model is good to a few per cent: another order has to promise more than that (eight
     // 1216x1216 frames: promised 2.7 % less, measured 0.8 % more)
-    const double margin = 0.96, limit_few = margin * given_us(few);
+    const double margin = 0.96, limit_few = margin * run_prefix(m, given, few);
     double best = few == many ? limit_few : 0.0;
     std::vector<double> best_key;
     auto offer = [&](double rate, double stagger, double lead, double stretch) {
@@ -216,7 +232,7 @@ std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>&
         double us = m.run(topological(t, deps, key, few));
         if (us >= limit_few) return;
         if (few < many) {
-            if (best == 0.0) best = margin * given_us(many);
+            if (best == 0.0) best = margin * run_prefix(m, given, many);
             us = m.run(topological(t, deps, key, many));
         }
         if (us < best) {

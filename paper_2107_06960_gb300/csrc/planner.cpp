@@ -312,9 +312,15 @@ void f32_shape(MafatStageDev& s, const Layer& L, const std::vector<TileInfo>& ti
     t.pack32_elems += (int64_t)s.n_nblk * s.f32_chunks * f32_chunk_channels(L.k) * L.k * L.k * s.n_blk;
 }
 
+constexpr int kMaxRings = 4;
+// What the 129 MB L2 keeps of a launch's data (measured, see build_plan): 81 MB of rings
+// and frames were kept, 104 MB were not.
+constexpr int64_t kL2Room = (int64_t)80 << 20;
+
 }  // namespace
 
-std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, bool* unsupported) {
+// build_plan with at most max_rings rings of tiles.
+static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rings, PlanTables& t, bool* unsupported) {
     *unsupported = false;
     const int n = (int)net.layers.size();
     t = PlanTables{};
@@ -649,9 +655,10 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
     t.slot_buf_elems = (buf + 127) / 128 * 128;  // 256-byte aligned for bf16, 512 for fp32
     // Several frames with a ring each, where that stays small, so that a frame's first tiles need
     // not wait for the last stages of the frame before: a frame's chain of layers is longer than
-    // the time its work keeps the SMs busy.  The limit keeps the rings in the 129 MB L2; an fp32
-    // plan's also in the 32 MiB area of the allocation-free call, next to the cut tensor, the outputs
-    // of the groups between and the counters, so that more rings never push a plan out of it.
+    // the time its work keeps the SMs busy.  The rings alone are held below the 129 MB L2 (with the
+    // frames' own data next to them: build_plan); an fp32 plan's also in the 32 MiB area of the
+    // allocation-free call, next to the cut tensor, the outputs of the groups between and the
+    // counters, so that more rings never push a plan out of it.
     const bool reorder = cfg.batch > 1 && !cfg.halo_reuse && !cfg.frame_major && cfg.ring_slots <= 0 && cfg.wave_tiles <= 0 &&
                          W >= max_tiles && S >= tiles_per_frame;
     // A ring of a whole frame gives each tile a slot of its own: a bf16 plan's slots are then as large
@@ -659,6 +666,7 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
     // second-group tile), so that more rings fit: four such frames 204 -> 170 us.  fp32 rings stay as
     // they were, so that the allocation-free call takes the plans that it took and no others.
     const bool own_slots = reorder && S == tiles_per_frame && cfg.dtype == 0;
+    bool crowded = false;  // bf16: the rings and the frames' own data are more than the L2 keeps
     if (reorder && S == tiles_per_frame) {
         int64_t set_elems = (int64_t)S * 2 * t.slot_buf_elems;
         if (own_slots) {
@@ -678,7 +686,9 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
             }
             limit = std::min<int64_t>((int64_t)16 << 20, ((int64_t)32 << 20) - others * 4 - 4096);
         }
-        t.ring_sets = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(cfg.batch, 4), limit / std::max<int64_t>(set_bytes, 1)));
+        t.ring_sets = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(cfg.batch, max_rings), limit / std::max<int64_t>(set_bytes, 1)));
+        const int64_t frames_bytes = (in_frame + (G > 1 ? cut_frame : 0) + out_frame) * cfg.batch * 2;
+        crowded = cfg.dtype == 0 && t.ring_sets > 1 && set_bytes * t.ring_sets + frames_bytes > kL2Room;
     }
     const int S_all = S * t.ring_sets;
     t.slot_off.assign(1, 0);
@@ -1004,8 +1014,11 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
     if (order.empty())
         for (int i = 0; i < (int)t.tasks.size(); ++i) order.push_back(i);
     if (reorder) {
-        order = hand_out_order(t, deps, order);
-        if (order.size() != t.tasks.size()) return "internal: the hand-out order lost a task";
+        std::vector<int> chosen = hand_out_order(t, deps, order);
+        if (chosen.size() != t.tasks.size()) return "internal: the hand-out order lost a task";
+        t.order_chosen = chosen != order;
+        order.swap(chosen);
+        if (crowded || max_rings < kMaxRings) t.crowded_us = modelled_us(t, deps, order, std::min(cfg.batch, 4 * kMaxRings));
     }
     {
         const int n_t = (int)t.tasks.size();
@@ -1103,6 +1116,29 @@ std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, boo
                                                                             cfg.grid_n[g], cfg.grid_m[g], 31.0, 2));
     }
     return validate_plan(net, t);
+}
+
+// Up to kMaxRings rings of tiles, and fewer where they crowd the L2 for nothing: what a ring and
+// the frames' input, cut tensor and output take beyond kL2Room is written to DRAM before it is
+// overwritten or read (16 608x608 frames, 71 MB of their own: 33, 136 and 225 MB written with two, three
+// and four rings of 22.7 MB, in 675, 677 and 677 us; 8 frames: 8, 55 and 91 MB in 359 us).  A
+// further ring is then kept only for a time that the order model sees: the fewest rings within
+// 2 % of the most (the 16 frames are modelled 0.6 % apart, the 8 frames 1.8 %; 32 416x416 frames
+// 3.5 %, of which 8 ran in 266 us with two rings and 246 with three, and four 608x608 frames 20 %:
+// 201 and 170 us).  Where all the rings leave the given order, one does.
+std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, bool* unsupported) {
+    std::string e = lower_plan(net, cfg, kMaxRings, t, unsupported);
+    if (!e.empty() || t.crowded_us <= 0.0) return e;
+    for (int rings = t.order_chosen ? 2 : 1; rings < t.ring_sets; ++rings) {
+        PlanTables fewer;
+        bool unsup = false;
+        if (!lower_plan(net, cfg, rings, fewer, &unsup).empty()) break;
+        if (fewer.crowded_us <= 1.02 * t.crowded_us) {
+            t = std::move(fewer);
+            break;
+        }
+    }
+    return "";
 }
 
 std::string validate_plan(const Net& net, const PlanTables& t) {

@@ -127,6 +127,8 @@ struct PlanTables {
     std::vector<MafatDepDev> deps;       // task dependency lists (halo reuse)
     int ring_slots = 0, wave_tiles = 0;
     int ring_sets = 1;                   // rings of ring_slots tiles: consecutive frames take turns
+    double crowded_us = 0.0;             // rings and frames' data over the L2's room: modelled time of the order (else 0)
+    bool order_chosen = false;           // the hand-out order is not the given one
     int n_counters = 0;                  // words after MAFAT_CTR_BASE
     int frame_ctr_base = 0;              // completion counters of every group but the last, per frame:
                                          // frame_ctr_base + frame * (n_groups - 1) + group
@@ -155,6 +157,8 @@ struct TaskDep {
 
 // The order in which the tasks are handed out (indices into t.tasks): `given`, or a better one.
 std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& given);
+// Modelled microseconds of the first `frames` frames of an order.
+double modelled_us(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& order, int frames);
 
 // Lower a configuration; returns "" or an error message.  `unsupported` is
 // set when the configuration is valid but not implemented.
