@@ -27,8 +27,8 @@
 // per pixel reading both operands from L1 took ~30 times as long), 1x1 256 -> 128 at 25; the
 // 16-layer network at 416x416 29.06 -> 0.83 ms, two 96x96 frames 53.9 -> 0.30 ms (the shapes'
 // choice and, for the two frames, the hand-out order included).  Those small frames are bound by
-// their chain of 12 dependent layers (10-45 us each: a 64-chunk item of one warp per scheduler
-// takes ~0.7 us a chunk).  Measured and not kept: the halo held twice in shared
+// their chain of 12 dependent layers (10-45 us each: a 64-chunk item of CT = 1, alone on its SM,
+// takes ~0.7 us a chunk; F32Cost in planner.h has the times of the other shapes).  Measured and not kept: the halo held twice in shared
 // memory so that pair instructions need no moves (42 instead of 50 TFLOP/s: 30 % more loads);
 // a chunk's rows unrolled (a lone warp's instruction fetches); 128 registers and 4 CTAs per SM.
 #include "sched.cuh"

@@ -266,18 +266,15 @@ int f32_region_items(const MafatStageDev& s, int ch, int cw) {
 
 // Shape of an fp32 stage's items.  A thread computes 8 pixels x f32_ct channels, the CTA's 128
 // threads f32_groups x 8 pixels x 8, 16, 32 or 64 channels.  With n items per SM, a stage takes
-// max(alone, n x full) per chunk of input channels: `alone` is what a chunk takes while an SM
-// has fewer than about three items (its schedulers then wait for one or two warps' instruction
-// fetches and loads), `full` what it adds once they are busy.  Both in microseconds, measured on
+// max(alone, n x full) per chunk of input channels: `alone` is what a chunk takes while the SMs
+// have fewer than about three items each (an item goes to the CTA that asks first, so some SMs run
+// three, which share its schedulers, while others have none), `full` what it adds once all have
+// three.  Both in microseconds, measured on
 // GB300 with single layers of 38x38 to 152x152 (256 -> 512 3x3, 512 -> 256 1x1); e.g. 3x3 38x38:
 // 96 items of ct 8 took 355 us, 192 of ct 4 187, 384 of ct 2 123, 768 of ct 1 144; 152x152:
 // 1077, 1117, 1393 and 1754 us.
-struct F32Cost {
-    int ct;
-    double alone, full;
-};
-const F32Cost kF32Cost3[] = {{8, 5.5, 1.8}, {4, 2.9, 1.0}, {2, 1.9, 0.62}, {1, 1.5, 0.4}};
-const F32Cost kF32Cost1[] = {{8, 2.5, 1.2}, {4, 1.7, 0.6}, {2, 1.2, 0.47}, {1, 0.8, 0.31}};
+const F32Cost kF32Cost3[] = {{8, 2.54, 5.5, 1.8}, {4, 1.42, 2.9, 1.0}, {2, 0.86, 1.9, 0.62}, {1, 0.58, 1.5, 0.4}};
+const F32Cost kF32Cost1[] = {{8, 1.05, 2.5, 1.2}, {4, 0.65, 1.7, 0.6}, {2, 0.45, 1.2, 0.47}, {1, 0.35, 0.8, 0.31}};
 
 void f32_shape(MafatStageDev& s, const Layer& L, const std::vector<TileInfo>& tiles, int l, const PlanConfig& cfg,
                int n_ctas, PlanTables& t) {
@@ -318,6 +315,12 @@ constexpr int kMaxRings = 4;
 constexpr int64_t kL2Room = (int64_t)80 << 20;
 
 }  // namespace
+
+const F32Cost& f32_cost(int k, int ct) {
+    const F32Cost* c = k == 3 ? kF32Cost3 : kF32Cost1;
+    while (c->ct != ct && c->ct > 1) ++c;
+    return *c;
+}
 
 // build_plan with at most max_rings rings of tiles.
 static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rings, PlanTables& t, bool* unsupported) {

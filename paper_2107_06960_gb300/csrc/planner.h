@@ -155,6 +155,19 @@ struct TaskDep {
     int bump_ctr = -1;     // (frame, group) counter this last stage of a group bumps
 };
 
+// Measured times of the fp32 kernel's chunks of input channels, microseconds, by the output channels
+// of a thread: of one item by itself (what a task's items take in the order model), and of a whole
+// stage (what its shape is chosen by, f32_shape).  Single layers on GB300, 3x3: a lone item 2.5, 1.1 to
+// 1.5, 0.7 to 1.1 and 0.6 to 0.8 us a chunk (8, 4, 2, 1 channels); with three on its SM 3.6 to 4.6, 1.8
+// to 2.4, 1.4 to 1.6 and 1.0, which is what a stage sees.
+struct F32Cost {
+    int ct;        // output channels per thread
+    double item;   // a chunk of an item that has its SM's schedulers to itself
+    double alone;  // a stage's time per chunk while the SMs have fewer than about three items each
+    double full;   // what a further item per SM adds to it beyond that
+};
+const F32Cost& f32_cost(int k, int ct);
+
 // The order in which the tasks are handed out (indices into t.tasks): `given`, or a better one.
 std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& given);
 // Modelled microseconds of the first `frames` frames of an order.
