@@ -145,8 +145,11 @@ typedef struct {
     int32_t wave_tiles;
     int32_t max_ctas;
     int32_t dtype;
-    int32_t frames_overlapped;  /* 1: the hand-out order overlaps frame f's second group with frame
-                                   f + 1's first (batch > 1, two groups, ring of a whole frame) */
+    int32_t frames_overlapped;  /* 1: frame f + 1's first group is handed out before the end of frame f's
+                                   second (two groups, batch > 1, ring of a whole frame): between its
+                                   stages, or all of it before, as the order model chose.  Plans of
+                                   one, three or four groups report 0, also where the order chosen
+                                   for a batch overlaps their frames */
     int32_t reserved;
 } mafat_plan_stats_t;
 

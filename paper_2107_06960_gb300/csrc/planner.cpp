@@ -996,14 +996,17 @@ static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rin
             while (pos < nx.size()) order.push_back(nx[pos++]);
         }
         if ((int)order.size() != n_t) return "internal: frame interleave lost a task";
-        t.frames_overlapped = 1;
+        t.frames_overlapped = 1;  // every candidate of hand_out_order overlaps them too
     }
     // Stages with many items (all tiles of one frame) keep every CTA busy whatever it holds,
     // so their CTAs take the next ticket early; stages with about a wave of items or fewer
     // take it only when the CTA can start it, so that no idle CTA waits for a busy one.
-    // With frames overlapped the next frame keeps every CTA busy in any stage, and the ticket is
-    // taken as soon as an item has its inputs (608x608: 16 frames 820 us so, 876 once the item's
-    // loads are out; one frame 94.4 and 93.1).
+    // With two groups' frames overlapped the next frame keeps every CTA busy in any stage, and the
+    // ticket is taken as soon as an item has its inputs (608x608: 16 frames 820 us so, 876 once the
+    // item's loads are out; one frame 94.4 and 93.1).  Batches of one group, or of more than two, keep
+    // one frame's threshold: taking every ticket early as well gains there in some and loses in
+    // others (eight 608x608 frames of one group 581 -> 571 us, a 75x101 block of three frames 59.2 -> 57.5, of
+    // 16 frames 274 -> 281).
     {
         const int64_t thr = cfg.lookahead_items > 0 ? cfg.lookahead_items
                             : t.frames_overlapped  ? 1
