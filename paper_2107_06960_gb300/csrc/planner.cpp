@@ -564,7 +564,6 @@ static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rin
             }
             s.w_off = t.weight_elems;
             t.weight_elems += (int64_t)s.n_nblk * s.n_chunks * s.n_bsteps * s.blob_elems;
-            t.weight32_elems += (int64_t)L.c_out * L.c_in * L.k * L.k;
             s.sb_off = (int)t.sb_elems;
             t.sb_elems += cout_pad;
             s.chain = chain_here ? 1 : 0;

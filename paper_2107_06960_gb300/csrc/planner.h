@@ -118,7 +118,6 @@ struct PlanTables {
     std::vector<MafatItemDev> items;
     std::vector<TmapReq> tmaps;          // index i = tensor map i (scratch inputs)
     int64_t weight_elems = 0;            // packed bf16 weight elements
-    int64_t weight32_elems = 0;          // fp32 weight elements
     int64_t pack32_elems = 0;            // fp32 weights as packed for the kernel (with padding)
     int64_t sb_elems = 0;                // scale / bias elements
     int64_t slot_buf_elems = 0;          // elements of the largest ping-pong buffer

@@ -424,7 +424,7 @@ mafat_status mafat_plan_ex(const mafat_net_t* net, int32_t n_groups, const int32
     p->cut_bytes = (size_t)t.cfg.batch * t.cut_c8 * 8 * t.cut_h * t.cut_w * p->esz;
     p->ctr_bytes = (size_t)(MAFAT_CTR_BASE + t.n_counters) * sizeof(uint32_t);
     p->scratch_bytes = t.scratch_elems * p->esz;
-    p->weight_bytes = (dt == MAFAT_BF16 ? t.weight_elems * 2 : t.weight32_elems * 4) + 2 * t.sb_elems * 4;
+    p->weight_bytes = (dt == MAFAT_BF16 ? t.weight_elems * 2 : t.pack32_elems * 4) + 2 * t.sb_elems * 4;
     if (p->dry_run) {
         *out = p;
         return MAFAT_OK;
