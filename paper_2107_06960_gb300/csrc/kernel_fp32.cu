@@ -452,17 +452,11 @@ cudaError_t mafat_launch_to_planar(const void* nhwc, void* planar, int frames, i
 int mafat_fp32_ctas_per_sm() { return kCtasPerSm; }
 size_t mafat_fp32_smem_bytes() { return (size_t)kSmemBytes; }
 
+cudaError_t mafat_prepare_fp32() {
+    return cudaFuncSetAttribute(mafat_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+}
+
 cudaError_t mafat_launch_fp32(const MafatKParams& p, int grid, cudaStream_t s) {
-    // more than 48 KB of dynamic shared memory is opted into once per device
-    static bool attr_set[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(mafat_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
-    }
     mafat_fp32_kernel<<<grid, kThreads, kSmemBytes, s>>>(p);
     return cudaGetLastError();
 }

@@ -1781,29 +1781,22 @@ __global__ void __launch_bounds__(128, 1)
 
 size_t mafat_tc_smem_bytes() { return (size_t)kSmemBytes; }
 
-namespace {
-template <bool kChain, bool kTrace>
-cudaError_t launch_tc(const MafatKParams& p, const CUtensorMap& in_map, int grid, cudaStream_t s) {
-    // the large dynamic shared memory is opted into once per device
-    static bool attr_set[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-        e = cudaFuncSetAttribute(mafat_tc_kernel<kChain, kTrace>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kSmemBytes);
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev] = true;
-    }
-    mafat_tc_kernel<kChain, kTrace><<<grid, kThreads, kSmemBytes, s>>>(p, in_map);
-    return cudaGetLastError();
+cudaError_t mafat_prepare_tc(bool chain, bool trace) {
+    auto opt_in = [](auto* kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes); };
+    if (chain) return trace ? opt_in(mafat_tc_kernel<true, true>) : opt_in(mafat_tc_kernel<true, false>);
+    return trace ? opt_in(mafat_tc_kernel<false, true>) : opt_in(mafat_tc_kernel<false, false>);
 }
-}  // namespace
 
 cudaError_t mafat_launch_tc(const MafatKParams& p, const CUtensorMap& in_map, int grid, bool chain, cudaStream_t s) {
-    const bool trace = p.trace != nullptr;
-    if (chain) return trace ? launch_tc<true, true>(p, in_map, grid, s) : launch_tc<true, false>(p, in_map, grid, s);
-    return trace ? launch_tc<false, true>(p, in_map, grid, s) : launch_tc<false, false>(p, in_map, grid, s);
+    if (chain && p.trace)
+        mafat_tc_kernel<true, true><<<grid, kThreads, kSmemBytes, s>>>(p, in_map);
+    else if (chain)
+        mafat_tc_kernel<true, false><<<grid, kThreads, kSmemBytes, s>>>(p, in_map);
+    else if (p.trace)
+        mafat_tc_kernel<false, true><<<grid, kThreads, kSmemBytes, s>>>(p, in_map);
+    else
+        mafat_tc_kernel<false, false><<<grid, kThreads, kSmemBytes, s>>>(p, in_map);
+    return cudaGetLastError();
 }
 
 cudaError_t mafat_launch_diag_umma(const void* a, const void* b, float* d, int n, int a_tmem, cudaStream_t s) {

@@ -40,9 +40,12 @@ struct MafatKParams {
 // bf16 tensor-core kernel (tcgen05 + TMA): one launch runs a whole plan; `chain` selects the
 // instance with the on-chip 3x3 -> 1x1 chaining path (plans that have chain stages).
 cudaError_t mafat_launch_tc(const MafatKParams& p, const CUtensorMap& in_map, int grid, bool chain, cudaStream_t s);
+// Opts the instance into its shared memory (more than 48 KB) on the current device; before its launches.
+cudaError_t mafat_prepare_tc(bool chain, bool trace);
 size_t mafat_tc_smem_bytes();
 // fp32 CUDA-core kernel: same task list, same scheduler.
 cudaError_t mafat_launch_fp32(const MafatKParams& p, int grid, cudaStream_t s);
+cudaError_t mafat_prepare_fp32();
 int mafat_fp32_ctas_per_sm();
 size_t mafat_fp32_smem_bytes();
 // NHWC [frames][h][w][c] -> octet-planar [frames][c8][h][w][8] (padded channels zero),

@@ -445,6 +445,8 @@ mafat_status mafat_plan_ex(const mafat_net_t* net, int32_t n_groups, const int32
         delete p;
         return cuda_fail(ee, what);
     };
+    e = dt == MAFAT_BF16 ? mafat_prepare_tc(p->has_chain, o.trace != 0) : mafat_prepare_fp32();
+    if (e != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
     if (dt == MAFAT_BF16) {
         std::vector<MafatItemRec> recs;
         mafat::build_records(t, recs);
