@@ -221,7 +221,7 @@ struct MafatEpiRec {
 // What the MMA issuer needs, packed in 32-bit words that it reads with three 16-byte
 // shared-memory loads and broadcasts word by word (the read is on the MMA warp's path between
 // items, while the tensor core keeps shared memory busy with its operands):
-//   w[0] key: stage * 256 + channel block, identifies a resident weight set
+//   w[0] key: stage << 15 | channel block, identifies a resident weight set
 //   w[1] sb: offset of the item's first channel in the scale / bias arrays
 //   w[2] bytes of one weight blob
 //   w[3] n_mid: MMA N of the item's (first) convolution

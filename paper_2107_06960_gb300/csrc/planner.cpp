@@ -1402,7 +1402,7 @@ void build_records(const PlanTables& t, std::vector<MafatItemRec>& out) {
             e.by0 = (int16_t)(it.by - e.bx0 * tk.nby);
         }
         uint32_t* w = r.mma.w;
-        w[0] = (uint32_t)(tk.stage * 256 + it.nb);
+        w[0] = (uint32_t)tk.stage << 15 | (uint32_t)it.nb;  // a layer may have more than 256 channel blocks
         w[1] = (uint32_t)(st.sb_off + it.nb * st.n_blk);
         w[2] = (uint32_t)(st.blob_elems * 2);
         w[3] = (uint32_t)st.n_blk;
