@@ -138,10 +138,14 @@ __device__ __forceinline__ void trace_put(unsigned long long* tr, int ticket, in
 // but the status word) for the next run on the same stream.
 __device__ __forceinline__ void finish_warp(uint32_t* ctr, int n_ctr, int lane) {
     uint32_t done = 0;
+    // The publications may be another lane's (elect.sync names no particular one) and the zeros are
+    // every lane's: the warp barriers put the ones before the release, the others after the acquire.
+    __syncwarp();
     if (lane == 0)  // release: this CTA's publications come first; acquire: so do the others'
         asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(done) : "l"(ctr + MAFAT_CTR_EXIT) : "memory");
     done = __shfl_sync(0xffffffffu, done, 0);
     if (done != gridDim.x - 1) return;
+    __syncwarp();
     for (int i = lane; i < n_ctr; i += 32)
         if (i != MAFAT_CTR_STATUS) ctr[i] = 0u;
 }
