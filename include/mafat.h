@@ -177,8 +177,9 @@ mafat_status mafat_set_weights(mafat_net_t* net, int32_t layer, const float* w_h
  * uses 1 or 2) layer groups split at the increasing cuts[0..n_groups-2] (the
  * first layer of each later group), group g tiled grid_n[g] x grid_m[g], for
  * `batch` images, in dtype dt.  The plan owns its device workspace (packed
- * weights, cut tensor, tile buffers, counters) on the current device; every
- * convolution must have weights set.  ENOFIT if a tile cannot be scheduled,
+ * weights, cut tensor, tile buffers, counters, and the work list: 256 bytes per
+ * item in BF16 plans, e.g. 0.6 MB for one 608x608 frame and 8.7 MB for 16) on the
+ * current device; every convolution must have weights set.  ENOFIT if a tile cannot be scheduled,
  * EUNSUPPORTED if a max-pool would be separated from its convolution.
  * Allocates device memory; not for use during stream capture. */
 mafat_status mafat_plan(const mafat_net_t* net, int32_t n_groups, const int32_t* cuts,

@@ -1,6 +1,7 @@
 // Plan tables shared by the host planner and the persistent kernels.
 //
-// A plan is lowered to three flat tables that live in device memory:
+// A plan is lowered to three flat tables (fp32 plans hold them in device memory; a bf16 plan's
+// are folded into one record per item, MafatItemRec):
 //   * MafatStageDev  -- one per fused convolution stage of the network (a conv
 //                       layer, with the 2x2/s2 max-pool that follows it folded
 //                       into its epilogue), with packed-weight offsets;
@@ -215,7 +216,7 @@ struct MafatEpiRec {
     int16_t pitch;           // flat stage: row pitch of the region (pixels); 0: 16x8 blocks
     int16_t flat_by;         // flat stage: the item's first block in the region
     int16_t by0, bx0;        // per-block-halo item: block row and column of its first block in the task
-    int32_t reserved[3];
+    int32_t reserved[3];     // fills the record to 96 bytes
 };
 
 // What the MMA issuer needs, packed in 32-bit words that it reads with three 16-byte
@@ -265,7 +266,7 @@ struct MafatLoadRec {
     int16_t chunk8;          // input octets per chunk (third coordinate step)
     int16_t lookahead;       // MafatStageDev::lookahead
     int16_t g_nby, g_by;     // gather item: block rows of its task, first block of the item
-    int16_t g_pad, g_k;      // gather item: reserved, kernel size
+    int16_t reserved, g_k;   // unused; gather item: kernel size
     int32_t g_cin;           // gather item: channels of the image
 };
 

@@ -1140,8 +1140,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                     ++a_cnt;
                     // the pieces that start inside this chunk (piece pc starts at blob pc * bpp);
-                    // no division: on this single thread, a runtime modulo per blob cost ~1.5 us
-                    // per chunk of a 3x3 256->512 item
+                    // no division: a runtime modulo per blob cost ~1.5 us per chunk of a 3x3
+                    // 256->512 item
 #pragma unroll 1
                     while (next_pc < P && next_pc * bpp < (c + 1) * n_bsteps) {
                         MAFAT_LOAD_PIECE(next_pc);

@@ -17,7 +17,7 @@ struct MafatKParams {
     int32_t pad0;
     const CUtensorMap* tmaps;     // scratch-input and cut tensor maps (bf16 path)
     const uint16_t* w_bf16;       // packed tensor-core weights
-    const float* w_f32;           // fp32 weights [cout][cin][k][k] per stage
+    const float* w_f32;           // fp32 weights as packed for the kernel (MafatStageDev::f32_w_off)
     const float* scale;
     const float* bias;
     const void* user_in;
@@ -30,7 +30,7 @@ struct MafatKParams {
     int64_t timeout_ns;
     unsigned long long* trace;    // per-item timestamps (null: off)
     // Regions every CTA warms into L2 (its 1/grid share of each) at start: the input, the
-    // packed weights, the work tables and the scale / bias arrays (bytes 0: unused slot).
+    // packed weights, the item records and the scale / bias arrays (bytes 0: unused slot).
     const void* pf_ptr[MAFAT_PF_REGIONS];
     int64_t pf_bytes[MAFAT_PF_REGIONS];
     int64_t pf_per[MAFAT_PF_REGIONS];   // each CTA's share of region r (bytes, multiple of 16)

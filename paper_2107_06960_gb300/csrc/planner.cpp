@@ -265,7 +265,7 @@ int f32_region_items(const MafatStageDev& s, int ch, int cw) {
 }
 
 // Shape of an fp32 stage's items.  A thread computes 8 pixels x f32_ct channels, the CTA's 128
-// threads f32_groups x 8 pixels x 8, 16, 32 or 64 channels.  With n items per SM, a stage takes
+// threads 16 groups of 8 pixels x 64, 32 or 16 channels (f32_ct 8, 4, 2) or 8 groups x 16 (f32_ct 1).  With n items per SM, a stage takes
 // max(alone, n x full) per chunk of input channels: `alone` is what a chunk takes while the SMs
 // have fewer than about three items each (an item goes to the CTA that asks first, so some SMs run
 // three, which share its schedulers, while others have none), `full` what it adds once all have

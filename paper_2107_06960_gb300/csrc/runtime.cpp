@@ -461,7 +461,7 @@ mafat_status mafat_plan_ex(const mafat_net_t* net, int32_t n_groups, const int32
         if ((e = cudaMemcpy(p->d_stages, t.stages.data(), t.stages.size() * sizeof(MafatStageDev), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
         if ((e = cudaMemcpy(p->d_tasks, t.tasks.data(), t.tasks.size() * sizeof(MafatTaskDev), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
         if ((e = cudaMemcpy(p->d_items, t.items.data(), t.items.size() * sizeof(MafatItemDev), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "cudaMemcpy");
-                }
+    }
     if (!t.deps.empty()) {
         if ((e = dalloc(p, &p->d_deps, t.deps.size() * sizeof(MafatDepDev))) != cudaSuccess) return bail(e, "cudaMalloc");
         if ((e = cudaMemcpy(p->d_deps, t.deps.data(), t.deps.size() * sizeof(MafatDepDev), cudaMemcpyHostToDevice)) !=

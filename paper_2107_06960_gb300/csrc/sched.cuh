@@ -9,8 +9,8 @@
 // trip: its grid is never larger than the SMs, one CTA each, so that all of its
 // CTAs run from the start.)  Waits are bounded
 // by a wall-clock limit: when it runs out the kernel records
-// MAFAT_DEV_TIMEOUT, raises the abort word and every later wait returns at
-// once, so the launch always ends.
+// MAFAT_DEV_TIMEOUT and raises the abort word, which every wait that has to
+// poll looks at every 16 polls, so the launch always ends.
 #pragma once
 #include "../../include/mafat.h"
 #include "kernels.h"

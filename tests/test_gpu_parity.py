@@ -204,9 +204,9 @@ def test_bf16_flat_blocks_random_shapes(mf):
 
 
 def test_fp32_flat_blocks_match_rectangles_and_oracle(mf):
-    # a 3x3, a 1x1 and a 3x3 on 2x2 tiles of 38x38: 20, 20 and 19-pixel regions run
-    # flattened (pitch 24), the later ones from the tile buffers of the scratch ring, in the
-    # fp32 check kernel as in the bf16 one
+    # a 3x3, a 1x1 and a 3x3 on 2x2 tiles of 38x38: 20, 20 and 19-pixel regions, the later ones
+    # from the tile buffers of the scratch ring; bf16 runs them flattened (pitch 24), fp32 in groups
+    # of 8 pixels row after row, and both in blocks with rect_blocks
     layers = [("conv", 3, 1, 1, 64), ("conv", 1, 1, 0, 32), ("conv", 3, 1, 1, 32)]
     assert (_issued(mf, layers, 38, 38, 16, None, [(2, 2)], mf.FP32) <
             _issued(mf, layers, 38, 38, 16, None, [(2, 2)], mf.FP32, rect_blocks=True))

@@ -177,7 +177,7 @@ def test_first_layer_k_steps(mf, c, k_issued):
     st = mf.Plan(net, None, [(1, 1)], dry_run=True).stats()
     assert st["issued_flops"] == 2 * (4 * 8 * 128) * 32 * k_issued
     assert st["executed_flops"] == 2 * 64 * 64 * 32 * c * 9
-    # the fp32 check mode has no tensor-core packing: issued = executed
+    # an fp32 plan of the same layer executes the same work
     st32 = mf.Plan(net, None, [(1, 1)], dtype=mf.FP32, dry_run=True).stats()
     assert st32["executed_flops"] == st["executed_flops"]
 
