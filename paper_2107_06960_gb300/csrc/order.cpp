@@ -54,8 +54,9 @@ struct Model {
     bool tc;
     int n_ctas;
 
-    // Makespan of the tasks in `order` (others are taken as absent).
-    double run(const std::vector<int>& order) const {
+    // Makespan of the tasks in `order` (others are taken as absent); start_of and end_of, where wanted,
+    // get when a task's first item could start and when its last one was published.
+    double run(const std::vector<int>& order, std::vector<double>* start_of = nullptr, std::vector<double>* end_of = nullptr) const {
         struct Cta {
             double mma_free = 0, mma_prev = 0, epi_free = 0, epi_prev = 0;
         };
@@ -92,6 +93,7 @@ struct Model {
             for (int k = 0; k < t.tasks[ti].n_items; ++k) {
                 Cta& q = cta[take[0].cta];
                 const double dep = std::max(take[0].at + (tc ? 1.7 : 2.5), ready + 0.5);
+                if (start_of && k == 0) (*start_of)[ti] = dep;
                 double out, next;
                 if (tc) {
                     const double load = std::max(dep, q.mma_prev) + c.load;  // two A stages
@@ -109,6 +111,7 @@ struct Model {
                 replace_top(next);
             }
             done[ti] = fin;
+            if (end_of) (*end_of)[ti] = fin;
             if (d.bump_ctr >= 0) group[d.bump_ctr] = std::max(group[d.bump_ctr], fin);
             end = std::max(end, fin);
         }
@@ -131,12 +134,11 @@ Model make_model(const PlanTables& t, const std::vector<TaskDep>& deps, std::vec
     return m;
 }
 
-// Modelled time of the tasks of the first frames, in the order given.
-double run_prefix(const Model& m, const std::vector<int>& order, int frames) {
+std::vector<int> prefix_of(const PlanTables& t, const std::vector<int>& order, int frames) {
     std::vector<int> prefix;
     for (int i : order)
-        if (m.t.tasks[i].frame < frames) prefix.push_back(i);
-    return m.run(prefix);
+        if (t.tasks[i].frame < frames) prefix.push_back(i);
+    return prefix;
 }
 
 // Topological order of the tasks with smallest key first.
@@ -172,9 +174,22 @@ std::vector<int> topological(const PlanTables& t, const std::vector<TaskDep>& de
 
 }  // namespace
 
-double modelled_us(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& order, int frames) {
-    std::vector<double> items;
-    return run_prefix(make_model(t, deps, items), order, frames);
+int rings_enough(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& order,
+                 const std::vector<int>& first, const std::vector<int>& last) {
+    const int n = (int)t.tasks.size(), frames = std::min(t.cfg.batch, 4 * t.ring_sets);
+    std::vector<double> items, start(n, 0.0), end(n, 0.0);
+    make_model(t, deps, items).run(prefix_of(t, order, frames), &start, &end);
+    std::vector<int> at(n);
+    for (int k = 0; k < n; ++k) at[order[k]] = k;
+    for (int rings = 2; rings < t.ring_sets; ++rings) {
+        bool same = true;
+        for (size_t q = (size_t)t.ring_slots * rings; q < first.size() && same; ++q) {
+            const int i = first[q], p = last[q - (size_t)t.ring_slots * rings];
+            same = at[p] < at[i] && (t.tasks[i].frame >= frames || end[p] + 0.5 <= start[i]);
+        }
+        if (same) return rings;
+    }
+    return t.ring_sets;
 }
 
 std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& given) {
@@ -227,7 +242,7 @@ std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>&
     };
     // the model is good to a few per cent: another order has to promise more than that (eight
     // 1216x1216 frames: promised 2.7 % less, measured 0.8 % more)
-    const double margin = 0.96, limit_few = margin * run_prefix(m, given, few);
+    const double margin = 0.96, limit_few = margin * m.run(prefix_of(t, given, few));
     double best = few == many ? limit_few : 0.0;
     std::vector<double> best_key;
     auto offer = [&](double rate, double stagger, double lead, double stretch) {
@@ -235,7 +250,7 @@ std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>&
         double us = m.run(topological(t, deps, key, few));
         if (us >= limit_few) return;
         if (few < many) {
-            if (best == 0.0) best = margin * run_prefix(m, given, many);
+            if (best == 0.0) best = margin * m.run(prefix_of(t, given, many));
             us = m.run(topological(t, deps, key, many));
         }
         if (us < best) {

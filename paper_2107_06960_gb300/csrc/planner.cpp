@@ -322,8 +322,9 @@ const F32Cost& f32_cost(int k, int ct) {
     return *c;
 }
 
-// build_plan with at most max_rings rings of tiles.
-static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rings, PlanTables& t, bool* unsupported) {
+// build_plan with at most max_rings rings of tiles, in the order given (empty: chosen here).
+static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rings, const std::vector<int>& given_order,
+                              PlanTables& t, bool* unsupported) {
     *unsupported = false;
     const int n = (int)net.layers.size();
     t = PlanTables{};
@@ -763,7 +764,7 @@ static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rin
 
     // ---- tasks in hand-out order, with their dependencies expressed as task indices
     std::vector<TaskDep> deps;
-    std::vector<int> last_task_of_seq;
+    std::vector<int> first_task_of_seq, last_task_of_seq;
     int seq = 0;
     for (int f = 0; f < cfg.batch; ++f) {
         for (int g = 0; g < G; ++g) {
@@ -915,6 +916,7 @@ static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rin
                             d.prev_task = prev_of_tile[qi];
                         }
                         if (g + 1 < G && s_out == t.stage_last[g]) d.bump_ctr = f * (G - 1) + g;
+                        if (s == t.stage_first[g]) first_task_of_seq.push_back((int)t.tasks.size());
                         prev_of_tile[qi] = (int)t.tasks.size();
                         t.tasks.push_back(tk);
                         deps.push_back(d);
@@ -1019,11 +1021,12 @@ static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rin
     if (order.empty())
         for (int i = 0; i < (int)t.tasks.size(); ++i) order.push_back(i);
     if (reorder) {
-        std::vector<int> chosen = hand_out_order(t, deps, order);
-        if (chosen.size() != t.tasks.size()) return "internal: the hand-out order lost a task";
-        t.order_chosen = chosen != order;
-        order.swap(chosen);
-        if (crowded || max_rings < kMaxRings) t.crowded_us = modelled_us(t, deps, order, std::min(cfg.batch, 4 * kMaxRings));
+        order = given_order.empty() ? hand_out_order(t, deps, order) : given_order;
+        if (order.size() != t.tasks.size()) return "internal: the hand-out order lost a task";
+        if (crowded && given_order.empty()) {
+            t.rings_enough = rings_enough(t, deps, order, first_task_of_seq, last_task_of_seq);
+            t.order = order;
+        }
     }
     {
         const int n_t = (int)t.tasks.size();
@@ -1123,26 +1126,18 @@ static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rin
     return validate_plan(net, t);
 }
 
-// Up to kMaxRings rings of tiles, and fewer where they crowd the L2 for nothing: what a ring and
-// the frames' input, cut tensor and output take beyond kL2Room is written to DRAM before it is
-// overwritten or read (16 608x608 frames, 71 MB of their own: 33, 136 and 225 MB written with two, three
-// and four rings of 22.7 MB, in 675, 677 and 677 us; 8 frames: 8, 55 and 91 MB in 359 us).  A
-// further ring is then kept only for a time that the order model sees: the fewest rings within
-// 2 % of the most (the 16 frames are modelled 0.6 % apart, the 8 frames 1.8 %; 32 416x416 frames
-// 3.5 %, of which 8 ran in 266 us with two rings and 246 with three, and four 608x608 frames 20 %:
-// 201 and 170 us).  Where all the rings leave the given order, one does.
+// Up to kMaxRings rings of tiles, and fewer where they crowd the L2 for nothing: what the rings and the
+// frames' input, cut tensor and output take beyond kL2Room is written to DRAM before it is
+// overwritten or read (16 608x608 frames, 71 MB of their own: 136 and 225 MB written with three and four
+// rings of 22.7 MB, both in 677 us).  There the rings go that the order never makes a tile wait
+// for.  Only those: 97 plans that gave rings up so ran in 0.994 to 1.004 of their time with all of
+// them; rings that the model puts at 0.3 to 2 % cost up to 10 % (16 368x608 frames 577 -> 633 us).
 std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, bool* unsupported) {
-    std::string e = lower_plan(net, cfg, kMaxRings, t, unsupported);
-    if (!e.empty() || t.crowded_us <= 0.0) return e;
-    for (int rings = t.order_chosen ? 2 : 1; rings < t.ring_sets; ++rings) {
-        PlanTables fewer;
-        bool unsup = false;
-        if (!lower_plan(net, cfg, rings, fewer, &unsup).empty()) break;
-        if (fewer.crowded_us <= 1.02 * t.crowded_us) {
-            t = std::move(fewer);
-            break;
-        }
-    }
+    std::string e = lower_plan(net, cfg, kMaxRings, {}, t, unsupported);
+    if (!e.empty() || t.rings_enough == 0 || t.rings_enough >= t.ring_sets) return e;
+    PlanTables fewer;
+    bool unsup = false;
+    if (lower_plan(net, cfg, t.rings_enough, t.order, fewer, &unsup).empty()) t = std::move(fewer);
     return "";
 }
 

@@ -126,8 +126,8 @@ struct PlanTables {
     std::vector<MafatDepDev> deps;       // task dependency lists (halo reuse)
     int ring_slots = 0, wave_tiles = 0;
     int ring_sets = 1;                   // rings of ring_slots tiles: consecutive frames take turns
-    double crowded_us = 0.0;             // rings and frames' data over the L2's room: modelled time of the order (else 0)
-    bool order_chosen = false;           // the hand-out order is not the given one
+    std::vector<int> order;              // the hand-out order, as indices of the tasks in lowering order
+    int rings_enough = 0;                // rings and frames' data over the L2's room: rings that do for the order (else 0)
     int n_counters = 0;                  // words after MAFAT_CTR_BASE
     int frame_ctr_base = 0;              // completion counters of every group but the last, per frame:
                                          // frame_ctr_base + frame * (n_groups - 1) + group
@@ -169,8 +169,10 @@ const F32Cost& f32_cost(int k, int ct);
 
 // The order in which the tasks are handed out (indices into t.tasks): `given`, or a better one.
 std::vector<int> hand_out_order(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& given);
-// Modelled microseconds of the first `frames` frames of an order.
-double modelled_us(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& order, int frames);
+// The fewest rings (at least two) with which the model runs `order` as it does with t.ring_sets: no tile
+// waits for its slot.  first / last: a tile's first and last task, tiles in order of their frames.
+int rings_enough(const PlanTables& t, const std::vector<TaskDep>& deps, const std::vector<int>& order,
+                 const std::vector<int>& first, const std::vector<int>& last);
 
 // Lower a configuration; returns "" or an error message.  `unsupported` is
 // set when the configuration is valid but not implemented.

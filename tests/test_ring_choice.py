@@ -1,5 +1,5 @@
 """How many rings of tile buffers a batched bf16 plan holds: up to four, but where the rings and the
-frames' own data are more than the L2 keeps, no more than the order model sees a use for."""
+frames' own data are more than the L2 keeps, none that the hand-out order has no use for."""
 import pytest
 
 import synth
@@ -15,10 +15,10 @@ def mf():
 
 @pytest.mark.parametrize("size,cut,grids,batch,rings", [
     (608, 8, [(5, 5), (2, 2)], 4, 4),      # four frames in lockstep need their four rings
-    (608, 8, [(5, 5), (2, 2)], 16, 2),     # two are as fast and stay in the L2
-    (608, 8, [(5, 5), (2, 2)], 64, 2),
+    (608, 8, [(5, 5), (2, 2)], 16, 3),     # no tile ever waits for the fourth
+    (608, 8, [(5, 5), (2, 2)], 64, 3),
     (416, 8, [(3, 3), (2, 2)], 8, 4),      # small enough beside the frames
-    (416, 8, [(3, 3), (2, 2)], 32, 3),     # too large, but the third ring is worth its time
+    (416, 8, [(3, 3), (2, 2)], 32, 3),
     (1216, 8, [(8, 8), (4, 4)], 8, 1),
 ])
 def test_rings_that_crowd_the_l2_need_a_reason(mf, size, cut, grids, batch, rings):
