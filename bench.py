@@ -46,7 +46,7 @@ def metric_of(name):
 DEFAULT_WORKLOAD = "yolo16_608_5x5_c8_2x2"
 L2_FLUSH_BYTES = 256 << 20
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
-KERNEL_SOURCES = ["kernel_tc.cu", "sched.cuh", "device_types.h", "planner.cpp"]
+KERNEL_SOURCES = ["kernel_tc.cu", "sched.cuh", "device_types.h", "planner.cpp", "order.cpp"]
 
 
 def kernel_source_hash():
