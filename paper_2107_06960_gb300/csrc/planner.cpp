@@ -1026,6 +1026,7 @@ static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rin
         if (crowded && given_order.empty()) {
             t.rings_enough = rings_enough(t, deps, order, first_task_of_seq, last_task_of_seq);
             t.order = order;
+            if (t.rings_enough < t.ring_sets) return "";  // build_plan lowers it again, with fewer
         }
     }
     {
@@ -1135,10 +1136,8 @@ static std::string lower_plan(const Net& net, const PlanConfig& cfg, int max_rin
 std::string build_plan(const Net& net, const PlanConfig& cfg, PlanTables& t, bool* unsupported) {
     std::string e = lower_plan(net, cfg, kMaxRings, {}, t, unsupported);
     if (!e.empty() || t.rings_enough == 0 || t.rings_enough >= t.ring_sets) return e;
-    PlanTables fewer;
-    bool unsup = false;
-    if (lower_plan(net, cfg, t.rings_enough, t.order, fewer, &unsup).empty()) t = std::move(fewer);
-    return "";
+    const std::vector<int> order = std::move(t.order);
+    return lower_plan(net, cfg, t.rings_enough, order, t, unsupported);
 }
 
 std::string validate_plan(const Net& net, const PlanTables& t) {
